@@ -187,7 +187,7 @@ struct ef_circuit {
 
     bool dirty = true;
     DBuf dWS, dWS32, dWSFF, dList, dListCount, dRecomp, dBits, dOut, dErr, dGradP, dGrad, dPbar, dSumP;
-    DBuf daT, daq, daq32, dalayer, damodes, dagpair, daPart, dCounters, daList;
+    DBuf daT, daq, daq32, dalayer, damodes, dagpair, daPart, dCounters, daList, daSamples, daImage;
     cudaStream_t own_stream = nullptr;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     bool timed = false;
@@ -206,7 +206,7 @@ struct ef_circuit {
     template <typename F> void for_each_buf(F f) {
         for (int b = 0; b < ef::kMaxBlocks; ++b) blk[b].for_each_buf(f);
         for (DBuf* d : {&dWS, &dWS32, &dWSFF, &dList, &dListCount, &dRecomp, &dBits, &dOut, &dErr, &dGradP, &dGrad, &dPbar, &dSumP, &daT,
-                        &daq, &daq32, &dalayer, &damodes, &dagpair, &daPart, &dCounters, &daList})
+                        &daq, &daq32, &dalayer, &damodes, &dagpair, &daPart, &dCounters, &daList, &daSamples, &daImage})
             f(*d);
     }
     ef_circuit() {
@@ -1464,9 +1464,7 @@ ef::ApproxDev approx_dev_for(const ef_circuit* c, const ef::ApproxDev& base, boo
         a.blk[b].P = fp64 ? B.dP64.p : B.dP32.p;
         a.blk[b].RC = fp64 ? B.dRC64.p : B.dRC32.p;
     }
-    a.kform = c->kform_ok ? 1 : 0;
-    const int eta_t = ef::approx_eta_template(a);
-    if (a.kform && ef::approx_smem_bytes(a, eta_t, fp64) > (size_t)200 * 1024) a.kform = 0;
+    ef::approx_choose_form(a, c->kform_ok, fp64);
     a.err_coef = fp64 ? 0.0 : base.err_coef;
     a.err_lin = fp64 ? 0.0 : base.err_lin;
     return a;
@@ -1491,8 +1489,10 @@ int approx_setup(ef_circuit* c, int64_t nb, int64_t t, uint64_t seed, uint64_t b
     a.gmodes = c->damodes.as<uint64_t>();
     a.gpair = c->dagpair.as<uint64_t>();
     a.R0 = c->R0;
-    a.key0 = (uint32_t)seed;
-    a.key1 = (uint32_t)(seed >> 32);
+    for (int r = 0; r < 10; ++r) {  // the key advances by two Weyl constants between rounds
+        a.rk0[r] = (uint32_t)seed + (uint32_t)r * 0x9E3779B9u;
+        a.rk1[r] = (uint32_t)(seed >> 32) + (uint32_t)r * 0xBB67AE85u;
+    }
     a.index_base = base;
     a.inactive0 = c->inactive[0];
     a.inactive1 = c->inactive[1];
@@ -1500,15 +1500,15 @@ int approx_setup(ef_circuit* c, int64_t nb, int64_t t, uint64_t seed, uint64_t b
     a.nb = nb;
     // enough (bitstring, chunk) items for about four waves of three CTAs per SM
     const int64_t sms = ef::sm_count();
+    a.sms = (int)sms;
     const int64_t target = sms * 3 * 4;
     int64_t chunks = std::max<int64_t>(1, (target + std::max<int64_t>(nb, 1) - 1) / std::max<int64_t>(nb, 1));
     chunks = std::min<int64_t>(chunks, std::max<int64_t>(1, t / 256));
     int64_t per = (t + chunks - 1) / chunks;
     per = (per + 127) / 128 * 128;
-    a.traj_per_cta = (int)std::min<int64_t>(per, (int64_t)1 << 30);
+    // (at most 2^25 trajectories per chunk: the samples of one must fit the workspace)
+    a.traj_per_cta = (int)std::min<int64_t>(per, (int64_t)1 << 25);
     a.n_chunks = (int)((t + a.traj_per_cta - 1) / a.traj_per_cta);
-    // one CTA per item (the hardware balances them); the listed FP64 redo strides
-    a.grid = (int)std::max<int64_t>(1, std::min<int64_t>(std::max<int64_t>(nb, 1) * a.n_chunks, 2147483647ll));
     a.kappa_max = 1e3;
     // K u, the per-trajectory bounds being in units of u = 2^-24. Calibrated
     // against FP64 on the same trajectories (eight circuits, 12,226 results: the
@@ -1575,6 +1575,43 @@ int approx_setup(ef_circuit* c, int64_t nb, int64_t t, uint64_t seed, uint64_t b
         a.blk[b].f = (int)B.pair_lm.size();
         a.blk[b].pair_lm = B.dPairLM.as<int>();
     }
+    // Workspace of a slab of items: samples (K form) and the bitstrings' images, for
+    // the FP32 pass and the FP64 redo alike, within 512 MiB (a slab of the 52-qubit
+    // LUCJ circuit is 880 bitstrings: several waves of the evaluation).
+    a.n_seg = (int)ef::approx_segments(a.traj_per_cta);
+    a.id_bits = a.k <= 256 ? 8 : 16;
+    {
+        // room for the entries of a segment: the expected number of trajectories with two or more
+        // flips and eight standard deviations (those past it are sampled again)
+        double p0 = 1.0, p1 = 0.0;
+        for (const CP& cp : c->cps) {
+            p1 = p1 * cp.pT0 + p0 * cp.pT1;
+            p0 *= cp.pT0;
+        }
+        const double mean = ef::approx_segment_traj() * std::max(0.0, 1.0 - p0 - p1);
+        a.ent_cap = (int)std::min<double>(ef::approx_segment_traj(), std::ceil(mean + 8.0 * std::sqrt(mean)) + 32.0);
+    }
+    const ef::ApproxDev first = approx_dev_for(c, a, fp64);
+    const ef::ApproxDev redo = c->opt.precision == EF_PREC_AUTO ? approx_dev_for(c, a, true) : first;
+    const int64_t img = std::max(first.img_bytes, redo.img_bytes);
+    size_t o_ent, o_sum, o_cnt;
+    const int64_t item = first.kform || redo.kform ? (int64_t)ef::approx_sample_bytes(a, 1, &o_ent, &o_sum, &o_cnt) : 0;
+    const int64_t budget = (int64_t)512 << 20, bytes = img + item * a.n_chunks;
+    const int64_t items = std::max<int64_t>(nb, 1) * a.n_chunks;
+    int64_t slab = bytes <= budget ? std::min<int64_t>(budget / bytes, 1 << 20) * a.n_chunks
+                                   : std::max<int64_t>(1, (budget - img) / std::max<int64_t>(item, 1));
+    slab = std::min(std::min(slab, items), std::max<int64_t>(1, 2147483647ll / a.n_seg));
+    a.slab_items = slab;
+    EF_CK(c->daSamples.ensure(item ? ef::approx_sample_bytes(a, slab, &o_ent, &o_sum, &o_cnt) : 0));
+    EF_CK(c->daImage.ensure((size_t)std::min<int64_t>(std::max<int64_t>(nb, 1), slab / a.n_chunks + 2) * img));
+    unsigned char* sp = c->daSamples.as<unsigned char>();
+    if (item) {
+        a.codes = reinterpret_cast<uint16_t*>(sp);
+        a.entries = reinterpret_cast<uint4*>(sp + o_ent);
+        a.hsums = reinterpret_cast<float*>(sp + o_sum);
+        a.seg_multi = reinterpret_cast<int*>(sp + o_cnt);
+    }
+    a.img = c->daImage.as<unsigned char>();
     a = approx_dev_for(c, a, fp64);
     return EF_OK;
 }
@@ -1599,7 +1636,6 @@ int approx_enqueue(ef_circuit* c, const ef::ApproxDev& a, const uint64_t* d_bits
         r.list = list;
         r.list_count = list_count;
         r.counters = a.counters + 4;  // the redo's own flips, LUs and rank-one minors
-        r.grid = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)a.grid, (int64_t)ef::sm_count() * 24));
         EF_CK(ef::launch_approx(r, d_bits, true, s, st));
         EF_CK(ef::launch_approx_finalize(r, d_out, d_se, d_err, nullptr, nullptr, true, s, st));
     }

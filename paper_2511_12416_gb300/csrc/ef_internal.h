@@ -122,7 +122,7 @@ struct ApproxDev {
     const uint64_t* gmodes;  // [kMaxBlocks][k]: local modes flipped in the block
     const uint64_t* gpair;   // [kMaxBlocks][k]: flippable pairs flipped in the block (K form)
     double R0;               // prod_j c_j / pT0_j
-    uint32_t key0, key1;
+    uint32_t rk0[10], rk1[10];  // Philox round keys
     uint64_t index_base;
     const uint64_t* gidx;    // null: bitstring i has global index index_base + i; else gidx[i]
     uint64_t inactive0, inactive1;
@@ -132,7 +132,20 @@ struct ApproxDev {
     const int* list_count;   //   their number (device)
     int traj_per_cta;
     int n_chunks;
-    int grid;                // CTAs (grid-stride over (bitstring, chunk) items)
+    // (bitstring, chunk) items run in slabs of slab_items; a launch covers the n_items from item0
+    int64_t slab_items, item0, n_items;
+    int sms;                 // SMs of the device
+    int pool;                // FP64: trajectories a warp pools
+    // K form: the sampled trajectories of a slab, per item four streams of n_seg segments: a code each
+    // (kSegTraj per segment), entries for those with two or more flips (ent_cap per segment, gate numbers
+    // of id_bits bits), and how many of these there are
+    int n_seg, ent_cap, id_bits;
+    uint16_t* codes;
+    uint4* entries;
+    int* seg_multi;
+    float* hsums;            // FP32: eight sums per thread over the small trajectories of an item
+    unsigned char* img;      // per bitstring of a slab: what the set-up leaves for the evaluation
+    int64_t img_bytes;
     int kform;               // 1: trajectory minors through K (every block has <= 64 flippable pairs)
     double kappa_max;        // A0 with ||A0||_1 ||A0^-1||_1 above this takes the rank-one form
     double err_coef;         // FP32 error estimate: K u32 (0: no estimate)
@@ -242,10 +255,14 @@ cudaError_t launch_grad(const GradDev& g, const uint64_t* bits, int64_t nb, cons
 size_t grad_minors_smem(int n, int eta, int L);
 cudaError_t launch_sum_rows(const double2* in, int64_t count, int64_t stride, int64_t width, double2* out,
                             cudaStream_t s, LaunchStats& st);
-// Raw Estimate: dynamic shared memory of one CTA; the launch over the items
+// Raw Estimate: K form or not and the bytes of a bitstring's image; bytes of
+// the samples of one item; the launch over the items
 // (all bitstrings, or a.list); the per-bitstring finalisation (listed: the
 // FP64 redo of the listed bitstrings; append_list collects flagged ones)
-size_t approx_smem_bytes(const ApproxDev& a, int eta_t, bool fp64);
+void approx_choose_form(ApproxDev& a, bool kform_ok, bool fp64);
+size_t approx_sample_bytes(const ApproxDev& a, int64_t items, size_t* entries, size_t* sums, size_t* counts);
+int64_t approx_segments(int64_t traj_per_cta);  // segments of an item's stream
+int approx_segment_traj();                      // trajectories of a segment
 int approx_eta_template(const ApproxDev& a);
 cudaError_t launch_approx(const ApproxDev& a, const uint64_t* bits, bool fp64, cudaStream_t s, LaunchStats& st);
 cudaError_t launch_approx_finalize(const ApproxDev& a, double* out, double* stderr_out, double* err_out,
