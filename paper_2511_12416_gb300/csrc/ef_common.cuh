@@ -306,6 +306,106 @@ __device__ __forceinline__ cplx_t<R> lu_det_regs(cplx_t<R> (&A)[N][N], R& er2, R
     return odd ? mk(-d.x, -d.y) : d;
 }
 
+// ---------------------------------------------------------------- FP32, Exact minors
+// The elimination of lu_det_regs<float, N> column by column (left-looking), bitwise
+// the same results: every entry meets the same multiply-adds in the same order and
+// the pivots are the same, but a column is read from the rows' memory only when
+// its turn comes. A row exchange then moves the row's multipliers and its offset
+// instead of the rest of its columns (392 selects at 8 x 8 instead of 672; with
+// the pivot comparisons they held the ALU at 59 % of its cycles and bound the
+// right-looking kernel), and only the multipliers and one column live in
+// registers: N (N - 1) + 3 N instead of 2 N^2. The updates are scalar: the packed
+// form wants each multiplier twice in a register pair.
+__device__ __forceinline__ float max3(float a, float b, float c) {
+#if defined(__CUDA_ARCH__) && (__CUDA_ARCH__ >= 1000)
+    float r;
+    asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+#else
+    return fmaxf(a, fmaxf(b, c));
+#endif
+}
+// Column K: rows ro[i] (offsets into M) in pivot order so far; the multipliers of
+// the finished rows k < K are those of the rows' places, L[i][k] for i > k.
+template <int N, int K>
+__device__ __forceinline__ void lu_column(const float2* __restrict__ M, int (&ro)[N], float2 (&L)[N][N], float2& d, bool& odd,
+                                          float& er2, float& pz, float& zc, int& nzero) {
+    if constexpr (K < N) {
+        float2 a[N];
+#pragma unroll
+        for (int i = 0; i < N; ++i) a[i] = M[ro[i] + K];
+        float cm2 = abs2(a[0]);
+#pragma unroll
+        for (int i = 1; i < N; i += 2) cm2 = i + 1 < N ? max3(cm2, abs2(a[i]), abs2(a[i + 1 < N ? i + 1 : i])) : fmaxf(cm2, abs2(a[i]));
+#pragma unroll
+        for (int k = 0; k < K; ++k)
+#pragma unroll
+            for (int i = k + 1; i < N; ++i) {
+                a[i].x = fmaf(L[i][k].y, a[k].y, fmaf(-L[i][k].x, a[k].x, a[i].x));
+                a[i].y = fmaf(-L[i][k].y, a[k].x, fmaf(-L[i][k].x, a[k].y, a[i].y));
+            }
+        float best = abs2(a[K]);
+        int p = K;
+#pragma unroll
+        for (int i = K + 1; i < N; ++i) {
+            const float m = abs2(a[i]);
+            const bool gt = m > best;
+            best = gt ? m : best;
+            p = gt ? i : p;
+        }
+        odd ^= (p != K);
+        // exchange rows K and p: this column, the multipliers, the offsets
+        const float2 old = a[K];
+        float2 Lo[N];
+#pragma unroll
+        for (int k = 0; k < K; ++k) Lo[k] = L[K][k];
+        const int oo = ro[K];
+#pragma unroll
+        for (int i = K + 1; i < N; ++i) {
+            const bool s = p == i;
+            a[K] = s ? a[i] : a[K];
+            a[i] = s ? old : a[i];
+            if (K + 1 < N) {
+#pragma unroll
+                for (int k = 0; k < K; ++k) {
+                    L[K][k] = s ? L[i][k] : L[K][k];
+                    L[i][k] = s ? Lo[k] : L[i][k];
+                }
+                ro[K] = s ? ro[i] : ro[K];
+                ro[i] = s ? oo : ro[i];
+            }
+        }
+        const float2 piv = a[K];
+        d = cmul(d, piv);
+        const bool nz = best >= min_pivot2(0.f);
+        const float inv = nz ? recip(best) : 0.f;
+        er2 += pivot_err_term(float(K + 1) * cm2 * inv);
+        pz *= nz ? best : 1.f;
+        zc = nz ? zc : float(K + 1) * cm2;
+        nzero += nz ? 0 : 1;
+        const float2 ip = mk(piv.x * inv, -piv.y * inv);
+#pragma unroll
+        for (int i = K + 1; i < N; ++i) L[i][K] = cmul(a[i], ip);
+        lu_column<N, K + 1>(M, ro, L, d, odd, er2, pz, zc, nzero);
+    }
+}
+// det of the N x N matrix whose row i starts at M + rows[i]
+template <int N>
+__device__ __forceinline__ float2 lu_det_columns(const float2* __restrict__ M, const int (&rows)[N], float& er2, float& zabs2) {
+    int ro[N];
+    float2 L[N][N];
+#pragma unroll
+    for (int i = 0; i < N; ++i) ro[i] = rows[i];
+    float2 d = mk(1.f, 0.f);
+    bool odd = false;
+    float pz = 1.f, zc = 0.f;
+    int nzero = 0;
+    er2 = 0.f;
+    lu_column<N, 0>(M, ro, L, d, odd, er2, pz, zc, nzero);
+    zabs2 = (nzero == 1) ? zc * pz : 0.f;
+    return odd ? mk(-d.x, -d.y) : d;
+}
+
 // The same elimination without the rounding-error proxy: for results that
 // are final (FP64) rather than estimated.
 template <typename R, int N, int K>
