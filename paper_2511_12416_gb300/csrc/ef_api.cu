@@ -186,7 +186,7 @@ struct ef_circuit {
     double R0 = 1.0;
 
     bool dirty = true;
-    DBuf dWS, dWS32, dWSFF, dList, dListCount, dRecomp, dBits, dOut, dErr, dGradP, dGrad, dPbar, dSumP;
+    DBuf dWS, dWS32, dWSFF, dList, dListCount, dRecomp, dDedup, dMarks, dBits, dOut, dErr, dGradP, dGrad, dPbar, dSumP;
     DBuf daT, daq, daq32, dalayer, damodes, dagpair, daPart, dCounters, daList, daSamples, daImage;
     cudaStream_t own_stream = nullptr;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
@@ -205,7 +205,7 @@ struct ef_circuit {
 
     template <typename F> void for_each_buf(F f) {
         for (int b = 0; b < ef::kMaxBlocks; ++b) blk[b].for_each_buf(f);
-        for (DBuf* d : {&dWS, &dWS32, &dWSFF, &dList, &dListCount, &dRecomp, &dBits, &dOut, &dErr, &dGradP, &dGrad, &dPbar, &dSumP, &daT,
+        for (DBuf* d : {&dWS, &dWS32, &dWSFF, &dList, &dListCount, &dRecomp, &dDedup, &dMarks, &dBits, &dOut, &dErr, &dGradP, &dGrad, &dPbar, &dSumP, &daT,
                         &daq, &daq32, &dalayer, &damodes, &dagpair, &daPart, &dCounters, &daList, &daSamples, &daImage})
             f(*d);
     }
@@ -874,9 +874,20 @@ struct ExactBuffers {
     int* list2;  // bitstrings still above tol after their listed determinants were redone
     int* count;  // [0] list size, [1] list2 size, [2 + B] listed determinants of block B
     int2* mlist[ef::kMaxBlocks];  // (column, pattern) of the determinants to redo in FP64
-    unsigned long long* recomp;   // [0] bitstrings, [1] determinants recomputed in FP64
+    unsigned long long* recomp;   // see ExactCombineDev
     int64_t cap;  // bitstrings per batch (row stride of the determinant buffers)
+    // equal bitstrings of a block factored once (dedup.table[0] null: each by itself)
+    ef::DedupDev dedup;
+    size_t dedup_clear;           // bytes from dedup.table[0] that are zeroed before every slice
+    uint32_t* marks;              // EF_PREC_AUTO: listed determinants per bitstring (see ExactCombineDev)
+    int mark_words;
 };
+
+// Equal bitstrings are looked for from this many bitstrings on. The search runs
+// beside the branch builder and costs a clearing of its table (about 2 us); 1500
+// uniform bitstrings of the 32-qubit workload, 6 % of them repeats on a block, just
+// pay for it.
+constexpr int64_t kDedupMin = 1024;
 
 // EF_PREC_AUTO redoes single determinants (rather than whole bitstrings) when
 // the thread-per-minor FP64 kernel covers every block and the combine can hold
@@ -990,6 +1001,16 @@ ef::ExactCombineDev make_combine(const ef_circuit* c, const ExactBuffers& eb) {
     cm.minors = 0;
     for (int b = 0; b < c->nblocks; ++b) cm.minors += (int64_t)1 << c->blk[b].r;
     cm.mcount = eb.count + 2;
+    if (c->opt.precision == EF_PREC_AUTO || eb.dedup.table[0]) cm.recomp = eb.recomp;
+    if (eb.dedup.table[0]) {
+        for (int b = 0; b < c->nblocks; ++b) {
+            cm.rep[b] = eb.dedup.rep[b];
+            cm.ucol[b] = eb.dedup.ucol[b];
+        }
+        cm.ucount = eb.dedup.ucount;
+        cm.marks = eb.marks;
+        cm.mark_words = eb.mark_words;
+    }
     cm.tol = c->opt.tol;
     cm.p_floor = c->p_floor;
     return cm;
@@ -1024,9 +1045,23 @@ void exact_account(ef_circuit* c, int64_t nb) {
     c->stats.dominant_kernel_flops = flops;
 }
 
-int exact_enqueue_build(ef_circuit* c, const ExactBuffers& eb, cudaStream_t s, ef::LaunchStats& st) {
+// Branch matrices, the counters cleared and, with a search table, the equal
+// bitstrings among the first nbb.
+int exact_enqueue_build(ef_circuit* c, const ExactBuffers& eb, const uint64_t* bits, int64_t nbb, cudaStream_t s,
+                        ef::LaunchStats& st) {
     const bool fp64_only = c->opt.precision == EF_PREC_FP64;
-    if (c->nblocks > 0) EF_CK(ef::launch_build_branches(eb.blk[0], eb.blk[1], c->nblocks, !fp64_only, s, st));
+    if (c->nblocks == 0) {
+        EF_CK(cudaMemsetAsync(eb.count, 0, 4 * sizeof(int), s));
+        EF_CK(cudaMemsetAsync(eb.recomp, 0, 4 * sizeof(unsigned long long), s));
+        return EF_OK;
+    }
+    ef::DedupDev d = eb.dedup;
+    d.bits = bits;
+    d.nb = nbb;
+    if (d.table[0]) EF_CK(cudaMemsetAsync(d.table[0], 0, eb.dedup_clear, s));
+    const bool counters = c->opt.precision == EF_PREC_AUTO || d.table[0];  // nothing else reads them
+    EF_CK(ef::launch_build_branches(eb.blk[0], eb.blk[1], c->nblocks, !fp64_only, counters ? eb.count : nullptr, eb.recomp,
+                                    d.table[0] ? &d : nullptr, s, st));
     return EF_OK;
 }
 
@@ -1054,8 +1089,9 @@ int exact_enqueue_lu(ef_circuit* c, const ExactBuffers& eb, const uint64_t* bits
 // per determinant when eb.mlist is set (FP32 pass -> listed determinants in
 // FP64 -> combine of the flagged bitstrings with a new estimate -> whole
 // bitstrings still above tol in FP64 -> their combine), else per bitstring.
+// cleared: eb.count is zero already (the first slice's, by the builder).
 int exact_enqueue_combine(ef_circuit* c, const ExactBuffers& eb, ef::ExactCombineDev cm, const uint64_t* bits,
-                          int64_t nbb, double* out, double* err, cudaStream_t s, ef::LaunchStats& st) {
+                          int64_t nbb, double* out, double* err, bool cleared, cudaStream_t s, ef::LaunchStats& st) {
     const bool autofix = c->opt.precision == EF_PREC_AUTO;
     cm.err_coef = fp32_err_coef(c);
     if (!autofix) {
@@ -1063,11 +1099,10 @@ int exact_enqueue_combine(ef_circuit* c, const ExactBuffers& eb, ef::ExactCombin
         return EF_OK;
     }
     const bool per_minor = eb.mlist[0] != nullptr;
-    EF_CK(cudaMemsetAsync(eb.count, 0, 4 * sizeof(int), s));
+    if (!cleared) EF_CK(cudaMemsetAsync(eb.count, 0, 4 * sizeof(int), s));
     for (int b = 0; b < c->nblocks; ++b) cm.mlist[b] = per_minor ? eb.mlist[b] : nullptr;
     EF_CK(ef::launch_exact_combine(cm, bits, nbb, nbb, nullptr, nullptr, out, err, eb.list, eb.count, s, st));
     for (int b = 0; b < c->nblocks; ++b) cm.mlist[b] = nullptr;
-    cm.recomp = eb.recomp;
     if (per_minor) {
         if (c->nblocks == 2 && eb.blk[0].eta == eb.blk[1].eta) {
             EF_CK(ef::launch_exact_lu_redo_minors(eb.blk[0], eb.blk[1], 2, bits, eb.mlist[0], eb.mlist[1],
@@ -1089,6 +1124,7 @@ int exact_enqueue_combine(ef_circuit* c, const ExactBuffers& eb, ef::ExactCombin
         cm.err_coef = 0.0;
         cm.src = 1;
         cm.count_full = 1;
+        cm.rep[0] = cm.rep[1] = nullptr;  // columns by place in the list
         EF_CK(ef::launch_exact_combine(cm, bits, nbb, nbb, eb.list2, eb.count + 1, out, err, nullptr, nullptr, s,
                                        st));
     } else {
@@ -1098,6 +1134,7 @@ int exact_enqueue_combine(ef_circuit* c, const ExactBuffers& eb, ef::ExactCombin
         cm.src = 1;
         cm.count_bits = 1;
         cm.count_full = 1;
+        cm.rep[0] = cm.rep[1] = nullptr;
         EF_CK(ef::launch_exact_combine(cm, bits, nbb, nbb, eb.list, eb.count, out, err, nullptr, nullptr, s, st));
     }
     return EF_OK;
@@ -1105,13 +1142,11 @@ int exact_enqueue_combine(ef_circuit* c, const ExactBuffers& eb, ef::ExactCombin
 
 int run_exact(ef_circuit* c, const ExactBuffers& eb, const uint64_t* d_bits, int64_t nb, double* d_out,
               double* d_err, cudaStream_t s, ef::LaunchStats& st) {
-    const bool autofix = c->opt.precision == EF_PREC_AUTO;
     exact_account(c, nb);
-    int rc = exact_enqueue_build(c, eb, s, st);
+    int rc = exact_enqueue_build(c, eb, d_bits, std::min(eb.cap, nb), s, st);
     if (rc) return rc;
     const ef::ExactCombineDev cm = make_combine(c, eb);
-    if (autofix) {
-        EF_CK(cudaMemsetAsync(eb.recomp, 0, 2 * sizeof(unsigned long long), s));
+    if (c->opt.precision == EF_PREC_AUTO || eb.dedup.table[0]) {
         c->last_recomp = eb.recomp;
         c->last_fp64_list_pending = 1;
     }
@@ -1119,13 +1154,20 @@ int run_exact(ef_circuit* c, const ExactBuffers& eb, const uint64_t* d_bits, int
     for (int64_t off = 0; off < nb; off += eb.cap) {
         const int64_t nbb = std::min(eb.cap, nb - off);
         const uint64_t* bits = d_bits + 2 * off;
+        if (off > 0 && eb.dedup.table[0]) {
+            ef::DedupDev d = eb.dedup;
+            d.bits = bits;
+            d.nb = nbb;
+            EF_CK(cudaMemsetAsync(d.table[0], 0, eb.dedup_clear, s));
+            EF_CK(ef::launch_dedup(eb.blk[0], eb.blk[1], d, s, st));
+        }
         if (c->timed && off == 0) EF_CK(cudaEventRecord(c->ev0, s));
         const int64_t before = st.launches;
         rc = exact_enqueue_lu(c, eb, bits, nbb, s, st);
         if (rc) return rc;
         lu_launches += st.launches - before;
         if (c->timed && off + nbb >= nb) EF_CK(cudaEventRecord(c->ev1, s));
-        rc = exact_enqueue_combine(c, eb, cm, bits, nbb, d_out + off, d_err ? d_err + off : nullptr, s, st);
+        rc = exact_enqueue_combine(c, eb, cm, bits, nbb, d_out + off, d_err ? d_err + off : nullptr, off == 0, s, st);
         if (rc) return rc;
     }
     c->stats.dominant_kernel_launches = lu_launches;
@@ -1135,7 +1177,7 @@ int run_exact(ef_circuit* c, const ExactBuffers& eb, const uint64_t* d_bits, int
 }
 
 // Workspace and device pointers of an Exact call with batches of `cap` bitstrings.
-int exact_buffers(ef_circuit* c, int64_t cap, ExactBuffers& eb) {
+int exact_buffers(ef_circuit* c, int64_t cap, bool dedup, ExactBuffers& eb) {
     const bool fp64_only = c->opt.precision == EF_PREC_FP64;
     eb = ExactBuffers{};
     eb.cap = cap;
@@ -1175,7 +1217,35 @@ int exact_buffers(ef_circuit* c, int64_t cap, ExactBuffers& eb) {
     eb.WSFF = c->dWSFF.as<float4>();
     EF_CK(c->dList.ensure(2 * (size_t)cap * sizeof(int)));
     EF_CK(c->dListCount.ensure(4 * sizeof(int)));
-    EF_CK(c->dRecomp.ensure(2 * sizeof(unsigned long long)));
+    EF_CK(c->dRecomp.ensure(4 * sizeof(unsigned long long)));
+    if (dedup) {
+        ef::DedupDev& d = eb.dedup;
+        uint32_t h = 1;
+        while ((int64_t)h < 2 * cap) h <<= 1;
+        d.hmask = h - 1;
+        EF_CK(c->dDedup.ensure(((size_t)2 * h + 4 + 4 * (size_t)cap) * sizeof(int) + (size_t)cap * 4 * sizeof(uint64_t)));
+        d.ubits[0] = c->dDedup.as<uint64_t>();
+        d.ubits[1] = d.ubits[0] + 2 * cap;
+        int* at = reinterpret_cast<int*>(d.ubits[1] + 2 * cap);
+        d.table[0] = at;
+        d.table[1] = at + h;
+        d.ucount = at + 2 * (size_t)h;
+        eb.dedup_clear = ((size_t)2 * h + 4) * sizeof(int);
+        at = d.ucount + 4;
+        for (int b = 0; b < 2; ++b) {
+            d.rep[b] = at + 2 * (size_t)b * cap;
+            d.ucol[b] = d.rep[b] + cap;
+            eb.blk[b].ubits = d.ubits[b];
+            eb.blk[b].ucount = d.ucount + b;
+            eb.blk[b].rep = d.rep[b];
+            eb.blk[b].ucol = d.ucol[b];
+        }
+        if (per_minor_recompute(c)) {
+            eb.mark_words = (int)((((int64_t)1 << c->blk[0].r) + ((int64_t)1 << c->blk[1].r) + 31) / 32);
+            EF_CK(c->dMarks.ensure((size_t)cap * eb.mark_words * sizeof(uint32_t)));
+            eb.marks = c->dMarks.as<uint32_t>();
+        }
+    }
     eb.list = c->dList.as<int>();
     eb.list2 = eb.list + cap;
     eb.count = c->dListCount.as<int>();
@@ -1196,7 +1266,7 @@ int exact_dev(ef_circuit* c, const uint64_t* d_bits, int64_t nb, double* d_out, 
     c->stats.logical_branch_dets = nb * (int64_t)std::ldexp(1.0, (int)c->cps.size());
     if (nb == 0) return EF_OK;
     ExactBuffers eb;
-    rc = exact_buffers(c, exact_batch(c, nb, (size_t)2 << 30), eb);
+    rc = exact_buffers(c, exact_batch(c, nb, (size_t)2 << 30), c->nblocks == 2 && nb >= kDedupMin, eb);
     if (rc) return rc;
     ef::LaunchStats st;
     return run_exact(c, eb, d_bits, nb, d_out, d_err, s, st);
@@ -1416,7 +1486,7 @@ int grad_dev(ef_circuit* c, const uint64_t* d_bits, int64_t nb, const double* d_
     EF_CK(c->dPbar.ensure((size_t)nb * ((size_t)1 << ksh) * sizeof(double2)));
     EF_CK(c->dSumP.ensure(((size_t)1 << ksh) * sizeof(double2)));
     g.pbar = c->dPbar.as<double2>();
-    if (c->nblocks > 0) EF_CK(ef::launch_build_branches(g.blk[0], g.blk[1], c->nblocks, false, s, st));
+    if (c->nblocks > 0) EF_CK(ef::launch_build_branches(g.blk[0], g.blk[1], c->nblocks, false, nullptr, nullptr, nullptr, s, st));
     for (int b = 0; b < c->nblocks; ++b) EF_CK(ef::launch_exact_lu_f64(g.blk[b], d_bits, nb, nullptr, nullptr, nb, s, st));
     if (c->timed) EF_CK(cudaEventRecord(c->ev0, s));
     EF_CK(ef::launch_grad(g, d_bits, nb, d_grad_p, d_out_p, s, st));
@@ -2070,10 +2140,15 @@ int ef_circuit_get_stats(ef_circuit* c, ef_stats* st) {
         c->stats.dominant_kernel_ms = ms;
     }
     if (c->last_mode == 1 && c->last_fp64_list_pending && c->last_recomp) {
-        unsigned long long cnt[2] = {0, 0};
+        unsigned long long cnt[4] = {0, 0, 0, 0};
         EF_CK(cudaMemcpy(cnt, c->last_recomp, sizeof(cnt), cudaMemcpyDeviceToHost));
         c->stats.fp64_recomputed = (int64_t)cnt[0];
         c->stats.executed_minor_lus += (int64_t)cnt[1];
+        for (int b = 0; b < c->nblocks; ++b) {  // minors that an equal bitstring's stood for
+            const int64_t spared = (int64_t)cnt[2 + b] << c->blk[b].r;
+            c->stats.executed_minor_lus -= spared;
+            c->stats.dominant_kernel_flops -= (double)spared * lu_flops(c->blk[b].eta);
+        }
         c->last_fp64_list_pending = 0;
     }
     if (c->last_mode == 2 && c->dCounters.p) {
@@ -2203,7 +2278,7 @@ size_t noalloc_layout(ef_circuit* c, int64_t nb, bool want32, unsigned char* bas
     eb.list = cv.take<int>((size_t)eb.cap);
     eb.list2 = cv.take<int>((size_t)eb.cap);
     eb.count = cv.take<int>(4);
-    eb.recomp = cv.take<unsigned long long>(2);
+    eb.recomp = cv.take<unsigned long long>(4);
     if (per_minor_recompute(c))
         for (int b = 0; b < c->nblocks; ++b)
             eb.mlist[b] = cv.take<int2>(((size_t)1 << c->blk[b].r) * (size_t)eb.cap);
@@ -2417,10 +2492,8 @@ int batch_enqueue(ef_batch* bt, cudaStream_t s, ef::LaunchStats& st) {
         ef_batch::Item& it = bt->items[i];
         if ((it.mode != 1 && it.mode != 2) || it.nb == 0) continue;
         ef_circuit* c = bt->cs[i];
-        int rc = exact_enqueue_build(c, it.eb, s, st);
+        int rc = exact_enqueue_build(c, it.eb, it.bits, std::min(it.nb, it.eb.cap), s, st);
         if (rc) return rc;
-        if (c->opt.precision == EF_PREC_AUTO)
-            EF_CK(cudaMemsetAsync(it.eb.recomp, 0, 2 * sizeof(unsigned long long), s));
     }
     for (size_t k = 0; k < bt->classes.size(); ++k) {
         int rc = batch_launch_queue(bt, (int)k, s, st);
@@ -2435,7 +2508,7 @@ int batch_enqueue(ef_batch* bt, cudaStream_t s, ef::LaunchStats& st) {
         cudaStream_t ss = bt->side[rr++ % ns];
         const ef::ExactCombineDev cm = make_combine(c, it.eb);
         if (it.mode == 1) {
-            int rc = exact_enqueue_combine(c, it.eb, cm, it.bits, it.nb, it.out, nullptr, ss, st);
+            int rc = exact_enqueue_combine(c, it.eb, cm, it.bits, it.nb, it.out, nullptr, true, ss, st);
             if (rc) return rc;
             continue;
         }
@@ -2444,7 +2517,7 @@ int batch_enqueue(ef_batch* bt, cudaStream_t s, ef::LaunchStats& st) {
             const int64_t nbb = std::min(it.eb.cap, it.nb - off);
             int rc = exact_enqueue_lu(c, it.eb, it.bits + 2 * off, nbb, ss, st);
             if (rc) return rc;
-            rc = exact_enqueue_combine(c, it.eb, cm, it.bits + 2 * off, nbb, it.out + off, nullptr, ss, st);
+            rc = exact_enqueue_combine(c, it.eb, cm, it.bits + 2 * off, nbb, it.out + off, nullptr, off == 0, ss, st);
             if (rc) return rc;
         }
     }
@@ -2588,7 +2661,7 @@ extern "C" int ef_batch_prob_dev(ef_batch* bt, const uint64_t* const* d_bits, co
             rc = begin_call(c, s, 1);
             if (rc) return rc;
             const int64_t cap = exact_batch(c, std::max<int64_t>(nb[i], 1), (size_t)2 << 30);
-            rc = exact_buffers(c, cap, it.eb);
+            rc = exact_buffers(c, cap, false, it.eb);
             if (rc) return rc;
             bool q = cap >= nb[i] && c->opt.precision != EF_PREC_FP64;
             for (int b = 0; b < c->nblocks; ++b) q = q && c->blk[b].eta <= ef::kMaxEtaThread;
@@ -2639,7 +2712,7 @@ extern "C" int ef_batch_prob_dev(ef_batch* bt, const uint64_t* const* d_bits, co
     ef::LaunchStats st0;
     for (int i = 0; i < nc; ++i)
         if (bt->items[i].mode == 1 && bt->items[i].nb > 0) {
-            int rc = exact_enqueue_build(bt->cs[i], bt->items[i].eb, s, st0);
+            int rc = exact_enqueue_build(bt->cs[i], bt->items[i].eb, nullptr, 0, s, st0);
             if (rc) return rc;
         }
     for (size_t k = 0; k < bt->classes.size(); ++k) {

@@ -26,6 +26,7 @@
 #include <algorithm>
 #include <map>
 #include <mutex>
+#include <type_traits>
 #include <utility>
 
 #include "ef_common.cuh"
@@ -164,9 +165,73 @@ __device__ __forceinline__ float4 cf_of_d(double2 a) {
     return make_float4(rh, ih, (float)(a.x - (double)rh), (float)(a.y - (double)ih));
 }
 
-__global__ void __launch_bounds__(128) k_build_branches(ExactBlockDev B0, ExactBlockDev B1, int want32) {
+// Equal bitstrings of a block (equal on its modes) have equal minors for every
+// pattern: each is factored once. Of the 10^4 uniform bitstrings of the 32-qubit
+// workload 54 % are distinct on 8 of 16 modes; sets sampled from a state or built as
+// products of alpha and beta strings repeat far more. Which of the equal ones
+// stands for them depends on the order of arrival, the results do not.
+__device__ __forceinline__ void dedup_range(const ExactBlockDev& B0, const ExactBlockDev& B1, const DedupDev& D, int64_t first,
+                                            int64_t step) {
+    for (int64_t x = first; x < 2 * D.nb; x += step) {
+        const int blk = x >= D.nb ? 1 : 0;
+        const int64_t b = x - (blk ? D.nb : 0);
+        const uint64_t m0 = blk ? B1.mask0 : B0.mask0, m1 = blk ? B1.mask1 : B0.mask1;
+        const uint64_t w0 = D.bits[2 * b] & m0, w1 = D.bits[2 * b + 1] & m1;
+        // a multiplicative mix of both words; the table is at most half full
+        uint64_t h = (w0 * 0x9E3779B97F4A7C15ull) ^ (w1 * 0xC2B2AE3D27D4EB4Full);
+        h ^= h >> 32;
+        h *= 0x9E3779B97F4A7C15ull;
+        uint32_t at = (uint32_t)(h >> 32) & D.hmask;
+        int* tab = blk ? D.table[1] : D.table[0];
+        int* ucol = blk ? D.ucol[1] : D.ucol[0];
+        uint64_t* ubits = blk ? D.ubits[1] : D.ubits[0];
+        int r = (int)b;
+        for (uint32_t probe = 0; probe <= D.hmask; ++probe) {
+            const int old = atomicCAS(&tab[at], 0, (int)b + 1);
+            if (old == 0) {  // the first of its kind
+                const int u = atomicAdd(&D.ucount[blk], 1);
+                ucol[b] = u;
+                ubits[2 * u] = w0;
+                ubits[2 * u + 1] = w1;
+                break;
+            }
+            if ((D.bits[2 * (old - 1)] & m0) == w0 && (D.bits[2 * (old - 1) + 1] & m1) == w1) {
+                r = old - 1;
+                break;
+            }
+            at = (at + 1) & D.hmask;
+        }
+        (blk ? D.rep[1] : D.rep[0])[b] = r;
+    }
+}
+
+__global__ void __launch_bounds__(256) k_dedup(ExactBlockDev B0, ExactBlockDev B1, DedupDev D) {
+    cudaGridDependencySynchronize();  // see launch_pdl
+    dedup_range(B0, B1, D, (int64_t)blockIdx.x * blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x);
+}
+
+cudaError_t launch_dedup(const ExactBlockDev& b0, const ExactBlockDev& b1, const DedupDev& d, cudaStream_t s,
+                         LaunchStats& st) {
+    const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>((2 * d.nb + 255) / 256, (int64_t)sm_count() * 8));
+    st.launches += 1;
+    return launch_pdl(k_dedup, dim3((unsigned)blocks), dim3(256), 0, s, b0, b1, d);
+}
+
+struct NoDedup {};
+template <typename D>  // DedupDev (two mode blocks: blockIdx.y = 2 searches) or NoDedup
+__global__ void __launch_bounds__(128) k_build_branches(ExactBlockDev B0, ExactBlockDev B1, int want32, int* count,
+                                                        unsigned long long* recomp, D dedup) {
     cudaGridDependencySynchronize();  // see launch_pdl
     extern __shared__ double2 smb[];
+    if (count && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < 4) {
+        count[threadIdx.x] = 0;
+        recomp[threadIdx.x] = 0ull;
+    }
+    if constexpr (std::is_same<D, DedupDev>::value)
+        if (blockIdx.y == 2) {  // beside the builder, which is mostly latency
+            dedup_range(B0, B1, dedup, (int64_t)blockIdx.x * blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x);
+            return;
+        }
     const ExactBlockDev& B = blockIdx.y ? B1 : B0;
     const int n = B.n, eta = B.eta, ne = n * eta;
     const uint32_t ny = 1u << B.r;
@@ -254,8 +319,8 @@ __global__ void __launch_bounds__(128) k_build_branches(ExactBlockDev B0, ExactB
     }
 }
 
-cudaError_t launch_build_branches(const ExactBlockDev& b0, const ExactBlockDev& b1, int nblk, bool want32,
-                                  cudaStream_t s, LaunchStats& st) {
+cudaError_t launch_build_branches(const ExactBlockDev& b0, const ExactBlockDev& b1, int nblk, bool want32, int* count,
+                                  unsigned long long* recomp, const DedupDev* dedup, cudaStream_t s, LaunchStats& st) {
     if (nblk < 1 || nblk > 2) return cudaErrorInvalidValue;
     size_t smem = 0;
     uint32_t ny = 1;
@@ -266,13 +331,19 @@ cudaError_t launch_build_branches(const ExactBlockDev& b0, const ExactBlockDev& 
             smem = std::max(smem, (size_t)(2 * b.n * b.eta + b.n * b.n) * sizeof(float4) + (size_t)b.n * sizeof(int));
         ny = std::max(ny, 1u << b.r);
     }
-    cudaError_t e = raise_dynamic_smem((const void*)k_build_branches, smem);
-    if (e != cudaSuccess) return e;
-    const dim3 grid(std::min<uint32_t>(ny, (uint32_t)sm_count() * 16u), (unsigned)nblk);
-    const cudaError_t le = launch_pdl(k_build_branches, grid, dim3(128), smem, s, b0, nblk == 2 ? b1 : b0, want32 ? 1 : 0);
-    if (le != cudaSuccess) return le;
+    const ExactBlockDev& bb = nblk == 2 ? b1 : b0;
+    const unsigned gx = std::min<uint32_t>(ny, (uint32_t)sm_count() * 16u);
+    cudaError_t e;
     st.launches += 1;
-    return cudaGetLastError();
+    if (dedup) {
+        if (nblk != 2) return cudaErrorInvalidValue;
+        if ((e = raise_dynamic_smem((const void*)k_build_branches<DedupDev>, smem)) != cudaSuccess) return e;
+        return launch_pdl(k_build_branches<DedupDev>, dim3(gx, 3u), dim3(128), smem, s, b0, bb, want32 ? 1 : 0, count, recomp,
+                          *dedup);
+    }
+    if ((e = raise_dynamic_smem((const void*)k_build_branches<NoDedup>, smem)) != cudaSuccess) return e;
+    return launch_pdl(k_build_branches<NoDedup>, dim3(gx, (unsigned)nblk), dim3(128), smem, s, b0, bb, want32 ? 1 : 0, count,
+                      recomp, NoDedup{});
 }
 
 // ---------------------------------------------------------------- 2b. FP64, thread per minor
@@ -286,7 +357,8 @@ __global__ void __launch_bounds__(128) k_exact_lu_f64t(ExactBlockDev B, const ui
                                                        int64_t nb, const int* __restrict__ list,
                                                        const int* __restrict__ list_count, int64_t stride) {
     cudaGridDependencySynchronize();  // see launch_pdl
-    const int64_t count = list ? (int64_t)(*list_count) : nb;
+    const int64_t count = list ? (int64_t)(*list_count) : B.ubits ? (int64_t)*B.ucount : nb;
+    if (!list && B.ubits) bits = B.ubits;
     const int64_t total = count << B.r;
     const int n = B.n;
     for (int64_t item = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; item < total;
@@ -338,7 +410,8 @@ __global__ void __launch_bounds__(256) k_exact_lu_rows(ExactBlockDev B, const ui
     constexpr int GPW = 32 / G;
     const int64_t warp_global = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const int64_t count = list ? (int64_t)(*list_count) : nb;
+    const int64_t count = list ? (int64_t)(*list_count) : B.ubits ? (int64_t)*B.ucount : nb;
+    if (!list && B.ubits) bits = B.ubits;
     const int Y = 1 << B.c_log2;
     const int64_t total = count * (int64_t)B.n_chunks;
     const int n = B.n, eta = B.eta;
@@ -562,9 +635,10 @@ __global__ void __launch_bounds__(128) k_exact_lu_ffm(ExactBlockDev B0, ExactBlo
         if (valid && r == 0) {
             const float4 det = !ok ? make_float4(0.f, 0.f, 0.f, 0.f)
                                    : ((inv & 1) ? make_float4(-d.x, -d.y, -d.z, -d.w) : d);
-            const size_t o = dix(pos, (uint32_t)z, B.r);
+            // (bitstrings that share the determinant may both have listed it: the same bytes twice)
+            const size_t o = dix(det_column(B.rep, B.ucol, pos, pos), (uint32_t)z, B.r);
             reinterpret_cast<float4*>(B.D64)[o] = det;
-            B.E32[o] = kErrRedone;
+            if (!B.rep) B.E32[o] = kErrRedone;  // else marked per bitstring
         }
     }
 }
@@ -635,9 +709,14 @@ __device__ __forceinline__ double neg_abs_int(double x) {
 // Determinant z of block B for D column col, as the combine's source says. A
 // determinant redone for a marked FP32 entry is stored as a float pair
 // (re hi, im hi, re lo, im lo) in its D64 slot.
-__device__ __forceinline__ double2 det_at(const ExactCombineDev& C, int B, size_t idx) {
+__device__ __forceinline__ bool redone(const ExactCombineDev& C, int B, int64_t b, uint32_t z, uint16_t code) {
+    if (!C.rep[0]) return err_redone(code);
+    const uint32_t bit = (B ? 1u << C.r[0] : 0u) + z;
+    return (C.marks[b * C.mark_words + (bit >> 5)] >> (bit & 31)) & 1u;
+}
+__device__ __forceinline__ double2 det_at(const ExactCombineDev& C, int B, size_t idx, int64_t b, uint32_t z) {
     if (C.src == 1) return C.D64[B][idx];
-    if (C.src == 2 && err_redone(C.E32[B][idx])) {
+    if (C.src == 2 && redone(C, B, b, z, C.E32[B][idx])) {
         const float4 f = reinterpret_cast<const float4*>(C.D64[B])[idx];
         return make_double2((double)f.x + (double)f.z, (double)f.y + (double)f.w);
     }
@@ -645,8 +724,27 @@ __device__ __forceinline__ double2 det_at(const ExactCombineDev& C, int B, size_
     return make_double2((double)v.x, (double)v.y);
 }
 // the stored error term of an FP32 determinant (0 for a redone one)
-__device__ __forceinline__ float err_term(const ExactCombineDev& C, int B, size_t idx) {
-    return err_term_value(C.E32[B][idx]);
+__device__ __forceinline__ float err_term(const ExactCombineDev& C, int B, size_t idx, int64_t b, uint32_t z) {
+    const uint16_t code = C.E32[B][idx];
+    return C.src == 2 && redone(C, B, b, z, code) ? 0.f : err_term_value(code);
+}
+// Listing a bitstring's determinants: clear its marks, then set those of the listed ones.
+__device__ __forceinline__ void clear_marks(const ExactCombineDev& C, int64_t b, int tid, int nt) {
+    if (C.rep[0])
+        for (int i = tid; i < C.mark_words; i += nt) C.marks[b * C.mark_words + i] = 0u;
+}
+__device__ __forceinline__ void list_minor(const ExactCombineDev& C, int B, int64_t b, int z) {
+    C.mlist[B][atomicAdd(&C.mcount[B], 1)] = make_int2((int)b, z);
+    if (C.rep[0]) {
+        const uint32_t bit = (B ? 1u << C.r[0] : 0u) + (uint32_t)z;
+        atomicOr(&C.marks[b * C.mark_words + (bit >> 5)], 1u << (bit & 31));
+    }
+}
+
+// Once per primary pass: bitstrings that an equal one stood for (statistics).
+__device__ __forceinline__ void count_equal(const ExactCombineDev& C, const int* list, int64_t nb) {
+    if (!list && C.recomp && C.rep[0] && blockIdx.x == 0 && threadIdx.x < 2)
+        atomicAdd(&C.recomp[2 + threadIdx.x], (unsigned long long)(nb - C.ucount[threadIdx.x]));
 }
 
 // Butterfly over lane bit j of a value held one per lane: the lane whose
@@ -742,12 +840,15 @@ __global__ void __launch_bounds__(256, 3) k_exact_combine(ExactCombineDev C, con
         if (C.count_minors)
             for (int B = 0; B < C.nblocks; ++B) atomicAdd(&C.recomp[1], (unsigned long long)C.mcount[B]);
     }
+    count_equal(C, list, nb);
     const bool want_err = C.err_coef > 0.0;
     const bool emit = want_err && !list && C.mlist[0] != nullptr;
     const int voff1 = C.nblocks == 2 ? (1 << C.r[0]) : 0;
     for (int64_t pos = blockIdx.x; pos < count; pos += gridDim.x) {
         const int64_t b = list ? (int64_t)list[pos] : pos;
-        const int64_t col = C.col_by_index ? b : pos;  // column of D holding this bitstring's determinants
+        // columns of D holding this bitstring's determinants
+        const int64_t plain = C.col_by_index ? b : pos;
+        const int64_t cols[kMaxBlocks] = {det_column(C.rep[0], C.ucol[0], b, plain), det_column(C.rep[1], C.ucol[1], b, plain)};
         const uint64_t w0 = bits[2 * b], w1 = bits[2 * b + 1];
         bool ok = ((w0 & C.inactive0) == 0) && ((w1 & C.inactive1) == 0);
         for (int B = 0; B < C.nblocks; ++B)
@@ -768,14 +869,14 @@ __global__ void __launch_bounds__(256, 3) k_exact_combine(ExactCombineDev C, con
             // amp = sum_z Omega(z) det(z); C(z) = Omega(z)
             const int nz = 1 << C.r[0];
             for (int z = tid; z < nz; z += NT) {
-                const size_t idx = dix(col, (uint32_t)z, C.r[0]);
-                const double2 v = det_at(C, 0, idx);
+                const size_t idx = dix(cols[0], (uint32_t)z, C.r[0]);
+                const double2 v = det_at(C, 0, idx, b, (uint32_t)z);
                 const double2 w = C.Omega[0][z];
                 ar = fma(w.x, v.x, fma(-w.y, v.y, ar));
                 ai = fma(w.x, v.y, fma(w.y, v.x, ai));
                 if (want_err) {
                     const float2 w32 = C.Omega32[0][z];
-                    const float vt = fmaf(w32.x, w32.x, w32.y * w32.y) * err_term(C, 0, idx);
+                    const float vt = fmaf(w32.x, w32.x, w32.y * w32.y) * err_term(C, 0, idx, b, (uint32_t)z);
                     var += vt;
                     if (emit) smV[z] = vt;
                 }
@@ -786,7 +887,7 @@ __global__ void __launch_bounds__(256, 3) k_exact_combine(ExactCombineDev C, con
                 float4* GB = B ? G1 : G0;
                 const int nz = 1 << C.r[B];
                 for (int z = tid; z < nz; z += NT) {
-                    const float2 v = C.D32[B][dix(col, (uint32_t)z, C.r[B])];
+                    const float2 v = C.D32[B][dix(cols[B], (uint32_t)z, C.r[B])];
                     GB[z] = cf_from_f(v);
                 }
             }
@@ -814,7 +915,7 @@ __global__ void __launch_bounds__(256, 3) k_exact_combine(ExactCombineDev C, con
             for (int B = 0; B < 2; ++B) {
                 double2* FB = B ? F1 : F0;
                 const int nz = 1 << C.r[B];
-                for (int z = tid; z < nz; z += NT) FB[z] = det_at(C, B, dix(col, (uint32_t)z, C.r[B]));
+                for (int z = tid; z < nz; z += NT) FB[z] = det_at(C, B, dix(cols[B], (uint32_t)z, C.r[B]), b, (uint32_t)z);
             }
             __syncthreads();
             // forward transform (the last stage also multiplies by the transformed
@@ -849,7 +950,7 @@ __global__ void __launch_bounds__(256, 3) k_exact_combine(ExactCombineDev C, con
                     const int nl = B == 0 ? nl0 : nl1;
                     double sx = 0.0, sy = 0.0;
                     for (int zl = 0; zl < nl; ++zl) {
-                        const double2 v = det_at(C, B, dix(col, (uint32_t)zl ^ sB, C.r[B]));
+                        const double2 v = det_at(C, B, dix(cols[B], (uint32_t)zl ^ sB, C.r[B]), b, (uint32_t)zl ^ sB);
                         const double2 w = C.Omega[B][zl];
                         sx = fma(w.x, v.x, fma(-w.y, v.y, sx));
                         sy = fma(w.x, v.y, fma(w.y, v.x, sy));
@@ -892,7 +993,7 @@ __global__ void __launch_bounds__(256, 3) k_exact_combine(ExactCombineDev C, con
                         cx += t.x;
                         cy += t.y;
                     }
-                    const float vt = fmaf(cx, cx, cy * cy) * err_term(C, B, dix(col, (uint32_t)z, C.r[B]));
+                    const float vt = fmaf(cx, cx, cy * cy) * err_term(C, B, dix(cols[B], (uint32_t)z, C.r[B]), b, (uint32_t)z);
                     var += vt;
                     if (emit) smV[B * voff1 + z] = vt;
                 }
@@ -946,15 +1047,15 @@ __global__ void __launch_bounds__(256, 3) k_exact_combine(ExactCombineDev C, con
         if (emit) {
             __syncthreads();
             const double theta = s_theta;
-            if (theta >= 0.0)
+            if (theta >= 0.0) {
+                clear_marks(C, b, tid, NT);
+                __syncthreads();
                 for (int B = 0; B < C.nblocks; ++B) {
                     const int nz = 1 << C.r[B];
                     for (int z = tid; z < nz; z += NT)
-                        if ((double)smV[B * voff1 + z] > theta) {
-                            const int idx = atomicAdd(&C.mcount[B], 1);
-                            C.mlist[B][idx] = make_int2((int)pos, z);
-                        }
+                        if ((double)smV[B * voff1 + z] > theta) list_minor(C, B, b, z);
                 }
+            }
         }
         __syncthreads();
     }
@@ -993,6 +1094,7 @@ __global__ void __launch_bounds__(NT, 3) k_exact_combine_ffr(ExactCombineDev C, 
         if (C.count_minors)
             for (int B = 0; B < 2; ++B) atomicAdd(&C.recomp[1], (unsigned long long)C.mcount[B]);
     }
+    count_equal(C, list, nb);
     const bool want_err = C.err_coef > 0.0;
     const bool emit = want_err && !list && C.mlist[0] != nullptr;
     const float floor_f = (float)C.p_floor, tol_f = (float)C.tol, ec_f = (float)C.err_coef;
@@ -1001,7 +1103,8 @@ __global__ void __launch_bounds__(NT, 3) k_exact_combine_ffr(ExactCombineDev C, 
     int it = 0;
     for (int64_t pos = blockIdx.x; pos < count; pos += gridDim.x, ++it) {
         const int64_t b = list ? (int64_t)list[pos] : pos;
-        const int64_t col = C.col_by_index ? b : pos;  // column of D holding this bitstring's determinants
+        const int64_t plain = C.col_by_index ? b : pos;
+        const int64_t cols[kMaxBlocks] = {det_column(C.rep[0], C.ucol[0], b, plain), det_column(C.rep[1], C.ucol[1], b, plain)};
         const int buf = it & 1;
         float* base = reinterpret_cast<float*>(smF) + (size_t)buf * buf_words;
         float4* G0 = reinterpret_cast<float4*>(base);
@@ -1032,13 +1135,15 @@ __global__ void __launch_bounds__(NT, 3) k_exact_combine_ffr(ExactCombineDev C, 
             for (int i = 0; i < kWregMax; ++i) {
                 const int e = tid + NT * i;
                 if (e >= nz) break;
-                const size_t idx = dix(col, (uint32_t)e, C.r[B]);
+                const size_t idx = dix(cols[B], (uint32_t)e, C.r[B]);
                 const float2 d = C.D32[B][idx];
                 const uint16_t ec = C.E32[B][idx];
                 errt[B][i] = want_err ? err_term_value(ec) : 0.f;
                 float4 v = cf_from_f(d);
-                if (C.src == 2 && err_redone(ec))  // redone, stored as a float pair
+                if (C.src == 2 && redone(C, B, b, (uint32_t)e, ec)) {  // redone, stored as a float pair
                     v = reinterpret_cast<const float4*>(C.D64[B])[idx];
+                    errt[B][i] = 0.f;
+                }
                 for (int pass = 0; pass < 2; ++pass)
                     for (int j = 0; j < rl; ++j) {
                         v = lane_butterfly(v, j, (e >> j) & 1);
@@ -1156,10 +1261,12 @@ __global__ void __launch_bounds__(NT, 3) k_exact_combine_ffr(ExactCombineDev C, 
                 else hi = mid;
             }
             const float t = __uint_as_float(lo);
+            clear_marks(C, b, lane, 32);
+            __syncwarp();
             for (int B = 0; B < 2; ++B) {
                 const int nz = B ? n1 : n0;
                 for (int z = lane; z < nz; z += 32)
-                    if (!(V[B * n0 + z] <= t)) C.mlist[B][atomicAdd(&C.mcount[B], 1)] = make_int2((int)pos, z);
+                    if (!(V[B * n0 + z] <= t)) list_minor(C, B, b, z);
             }
         }
     }
@@ -1207,6 +1314,7 @@ __global__ void __launch_bounds__(128, (RL >= 5 ? 2 : 3)) k_exact_combine_wp(Exa
         if (C.count_minors)
             for (int B = 0; B < 2; ++B) atomicAdd(&C.recomp[1], (unsigned long long)C.mcount[B]);
     }
+    count_equal(C, list, nb);
     const bool want_err = C.err_coef > 0.0;
     const bool emit = want_err && !list && C.mlist[0] != nullptr;
     const float floor_f = (float)C.p_floor, tol_f = (float)C.tol, ec_f = (float)C.err_coef;
@@ -1230,7 +1338,6 @@ __global__ void __launch_bounds__(128, (RL >= 5 ? 2 : 3)) k_exact_combine_wp(Exa
     const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
     for (int64_t pos = (int64_t)blockIdx.x * (blockDim.x >> 5) + wib; pos < count; pos += nwarps) {
         const int64_t b = list ? (int64_t)list[pos] : pos;
-        const int64_t col = C.col_by_index ? b : pos;
         const uint64_t w0 = bits[2 * b], w1 = bits[2 * b + 1];
         bool ok = ((w0 & C.inactive0) == 0) && ((w1 & C.inactive1) == 0);
         for (int B = 0; B < 2; ++B)
@@ -1254,7 +1361,12 @@ __global__ void __launch_bounds__(128, (RL >= 5 ? 2 : 3)) k_exact_combine_wp(Exa
             // the row's NL determinants and error terms are contiguous and start at a
             // multiple of NL: read them as 16-byte (and, below 8 error terms, 4- or
             // 8-byte) vectors
-            const size_t base = dix(col, (uint32_t)z0, C.r[B]);
+            const size_t base = dix(det_column(C.rep[B], C.ucol[B], b, C.col_by_index ? b : pos), (uint32_t)z0, C.r[B]);
+            uint32_t marked = 0;  // redone patterns of the row (their values are float pairs)
+            if (C.src == 2 && C.rep[0]) {
+                const uint32_t bit = (B ? (uint32_t)n0 : 0u) + (uint32_t)z0;
+                marked = C.marks[b * C.mark_words + (bit >> 5)] >> (bit & 31);
+            }
             const float4* dv = reinterpret_cast<const float4*>(C.D32[B] + base);
             uint32_t ew[(NL + 1) / 2];
             if constexpr (NL >= 8) {
@@ -1277,8 +1389,10 @@ __global__ void __launch_bounds__(128, (RL >= 5 ? 2 : 3)) k_exact_combine_wp(Exa
                     const uint16_t ec = (uint16_t)(ew[l / 2] >> (16 * h));
                     errt[rr][l + h] = want_err ? err_term_value(ec) : 0.f;
                     v[l + h] = h ? make_float4(dd.z, dd.w, 0.f, 0.f) : make_float4(dd.x, dd.y, 0.f, 0.f);
-                    if (C.src == 2 && err_redone(ec))  // redone, stored as a float pair
+                    if (C.src == 2 && (((marked >> (l + h)) & 1u) || err_redone(ec))) {
                         v[l + h] = reinterpret_cast<const float4*>(C.D64[B])[base + l + h];
+                        errt[rr][l + h] = 0.f;
+                    }
                 }
             }
             row_wht<RL>(v, cf_add, cf_sub);
@@ -1402,12 +1516,14 @@ __global__ void __launch_bounds__(128, (RL >= 5 ? 2 : 3)) k_exact_combine_wp(Exa
                 else hi = mid;
             }
             const float t = __uint_as_float(lo);
+            clear_marks(C, b, lane, 32);
+            __syncwarp();
             for (int p = lane; p < n0 + n1; p += 32)
                 if (!(V[p] <= t)) {
                     const int B = p < n0 ? 0 : 1;
                     const int pz = B ? p - n0 : p, shB = C.r[B] - RL;
                     const int z = ((pz & ((1 << shB) - 1)) << RL) | (pz >> shB);  // back to (h, l)
-                    C.mlist[B][atomicAdd(&C.mcount[B], 1)] = make_int2((int)pos, z);
+                    list_minor(C, B, b, z);
                 }
         }
         __syncwarp();

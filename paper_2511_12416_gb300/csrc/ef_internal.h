@@ -47,6 +47,32 @@ struct ExactBlockDev {
     uint16_t* E32;          // FP32 LU: error term |det|^2 er2 + zabs2 as bfloat16 rounded up;
                             // the sign bit set marks a determinant redone in D64
     double2* D64;           // FP64 LU: det
+    // With equal bitstrings of the block factored once (else null): the distinct
+    // ones and their number; of every bitstring of the slice the index of the
+    // first equal one, and of that one its place among the distinct ones
+    const uint64_t* ubits;
+    const int* ucount;
+    const int* rep;
+    const int* ucol;
+};
+
+// Column of D32 / E32 / D64 that holds bitstring b's determinants of a block.
+__device__ __forceinline__ int64_t det_column(const int* rep, const int* ucol, int64_t b, int64_t plain) {
+    return rep ? (int64_t)ucol[rep[b]] : plain;
+}
+
+// Search for a slice's equal bitstrings, block by block: open addressing in a
+// table of hmask + 1 entries per block (index of a bitstring + 1, 0: free),
+// zeroed before the launch like ucount.
+struct DedupDev {
+    const uint64_t* bits;
+    int64_t nb;
+    uint32_t hmask;
+    int* table[kMaxBlocks];
+    int* rep[kMaxBlocks];
+    int* ucol[kMaxBlocks];
+    uint64_t* ubits[kMaxBlocks];
+    int* ucount;            // [kMaxBlocks]
 };
 
 // Index of the determinant of pattern z (of 2^r) for bitstring column col in
@@ -92,7 +118,16 @@ struct ExactCombineDev {
     // variance terms are large (mlist[B] entries (column, z), counts in mcount)
     int2* mlist[kMaxBlocks];
     int* mcount;
-    // recompute counters: [0] bitstrings, [1] FP64 determinants; the launch adds
+    // equal bitstrings factored once (see ExactBlockDev; null: columns as col_by_index says). A
+    // determinant then serves several bitstrings, and which of them wanted it redone is kept per
+    // bitstring: marks[b][mark_words], bit (2^r_0 of block 0, then block 1) z
+    const int* rep[kMaxBlocks];
+    const int* ucol[kMaxBlocks];
+    const int* ucount;
+    uint32_t* marks;
+    int mark_words;
+    // recompute counters: [0] bitstrings, [1] FP64 determinants, [2 + B] bitstrings of block B
+    // that an equal one stood for; the launch adds
     // the list size (count_bits), list size x minors (count_full), sum of mcount (count_minors)
     unsigned long long* recomp;
     int count_bits, count_full, count_minors;
@@ -221,9 +256,13 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
-// branch matrices of nblk (1 or 2) mode blocks in one launch
-cudaError_t launch_build_branches(const ExactBlockDev& b0, const ExactBlockDev& b1, int nblk, bool want32,
-                                  cudaStream_t s, LaunchStats& st);
+// branch matrices of nblk (1 or 2) mode blocks in one launch, which also clears
+// the call's counters (count[4], recomp[4]; null: none) and looks for equal
+// bitstrings (dedup; null: does not)
+cudaError_t launch_build_branches(const ExactBlockDev& b0, const ExactBlockDev& b1, int nblk, bool want32, int* count,
+                                  unsigned long long* recomp, const DedupDev* dedup, cudaStream_t s, LaunchStats& st);
+cudaError_t launch_dedup(const ExactBlockDev& b0, const ExactBlockDev& b1, const DedupDev& d, cudaStream_t s,
+                         LaunchStats& st);
 // FP32 minors of nblk (1 or 2) mode blocks with the same eta in one launch
 cudaError_t launch_exact_lu_f32(const ExactBlockDev& b0, const ExactBlockDev& b1, int nblk, const uint64_t* bits,
                                 int64_t nb, cudaStream_t s, LaunchStats& st);

@@ -40,6 +40,11 @@ __global__ void __launch_bounds__(128) k_exact_lu_f32(ExactBlockDev B0, ExactBlo
     // both mode blocks in one launch (blockIdx.z): one tail instead of two
     const ExactBlockDev& B = blockIdx.z ? B1 : B0;
     constexpr int S = ETA | 1;
+    if (B.ubits) {  // the distinct bitstrings of the block
+        bits = B.ubits;
+        nb = *B.ucount;
+        if ((int64_t)blockIdx.x * blockDim.x >= nb) return;
+    }
     const int n = B.n;
     const int Y = 1 << B.c_log2;
     const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
