@@ -136,10 +136,10 @@ struct HostBlock {
     // device
     DBuf dS0C, dT, dF, dOmega, dOmega32, dOmegaHat, dOmegaHatFF, dSh, dPerm, dGoff, dInvOff, dInvXs, dM64, dM32, dD32, dE32, dD64, dMlist,
         dP64, dP32, dRC64, dRC32, dCols, dPairLM;
-    DBuf dCot, dEbar, dTbar, dSbar, dSumT, dSumS, dSumE;
+    DBuf dCot, dEbar, dTbar, dSbar;
     template <typename F> void for_each_buf(F f) {
         for (DBuf* b : {&dS0C, &dT, &dF, &dOmega, &dOmega32, &dOmegaHat, &dOmegaHatFF, &dSh, &dPerm, &dGoff, &dInvOff, &dInvXs, &dM64, &dM32, &dD32, &dE32, &dD64, &dMlist, &dP64, &dP32, &dRC64,
-                        &dRC32, &dCols, &dPairLM, &dCot, &dEbar, &dTbar, &dSbar, &dSumT, &dSumS, &dSumE})
+                        &dRC32, &dCols, &dPairLM, &dCot, &dEbar, &dTbar, &dSbar})
             f(*b);
     }
     void release() {
@@ -186,7 +186,7 @@ struct ef_circuit {
     double R0 = 1.0;
 
     bool dirty = true;
-    DBuf dWS, dWS32, dWSFF, dList, dListCount, dRecomp, dDedup, dMarks, dBits, dOut, dErr, dGradP, dGrad, dPbar, dSumP;
+    DBuf dWS, dWS32, dWSFF, dList, dListCount, dRecomp, dDedup, dMarks, dBits, dOut, dErr, dGradP, dGrad, dPbar, dSums;
     DBuf daT, daq, daq32, dalayer, damodes, dagpair, daPart, dCounters, daList, daSamples, daImage;
     cudaStream_t own_stream = nullptr;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
@@ -205,7 +205,7 @@ struct ef_circuit {
 
     template <typename F> void for_each_buf(F f) {
         for (int b = 0; b < ef::kMaxBlocks; ++b) blk[b].for_each_buf(f);
-        for (DBuf* d : {&dWS, &dWS32, &dWSFF, &dList, &dListCount, &dRecomp, &dDedup, &dMarks, &dBits, &dOut, &dErr, &dGradP, &dGrad, &dPbar, &dSumP, &daT,
+        for (DBuf* d : {&dWS, &dWS32, &dWSFF, &dList, &dListCount, &dRecomp, &dDedup, &dMarks, &dBits, &dOut, &dErr, &dGradP, &dGrad, &dPbar, &dSums, &daT,
                         &daq, &daq32, &dalayer, &damodes, &dagpair, &daPart, &dCounters, &daList, &daSamples, &daImage})
             f(*d);
     }
@@ -1453,9 +1453,6 @@ int grad_dev(ef_circuit* c, const uint64_t* d_bits, int64_t nb, const double* d_
         EF_CK(B.dEbar.ensure((size_t)nb * ((size_t)1 << B.r_loc) * sizeof(double2)));
         EF_CK(B.dTbar.ensure(ny * std::max<size_t>(1, (size_t)B.L * B.n * B.n) * sizeof(double2)));
         EF_CK(B.dSbar.ensure(ny * ne * sizeof(double2)));
-        EF_CK(B.dSumT.ensure(std::max<size_t>(1, (size_t)B.L * B.n * B.n) * sizeof(double2)));
-        EF_CK(B.dSumS.ensure(ne * sizeof(double2)));
-        EF_CK(B.dSumE.ensure(((size_t)1 << B.r_loc) * sizeof(double2)));
         ef::ExactBlockDev& d = g.blk[b];
         exact_block_geometry(c, b, nb, d);
         d.S0C = B.dS0C.as<double2>();
@@ -1484,7 +1481,6 @@ int grad_dev(ef_circuit* c, const uint64_t* d_bits, int64_t nb, const double* d_
         g.sbar[b] = B.dSbar.as<double2>();
     }
     EF_CK(c->dPbar.ensure((size_t)nb * ((size_t)1 << ksh) * sizeof(double2)));
-    EF_CK(c->dSumP.ensure(((size_t)1 << ksh) * sizeof(double2)));
     g.pbar = c->dPbar.as<double2>();
     if (c->nblocks > 0) EF_CK(ef::launch_build_branches(g.blk[0], g.blk[1], c->nblocks, false, nullptr, nullptr, nullptr, s, st));
     for (int b = 0; b < c->nblocks; ++b) EF_CK(ef::launch_exact_lu_f64(g.blk[b], d_bits, nb, nullptr, nullptr, nb, s, st));
@@ -1492,29 +1488,43 @@ int grad_dev(ef_circuit* c, const uint64_t* d_bits, int64_t nb, const double* d_
     EF_CK(ef::launch_grad(g, d_bits, nb, d_grad_p, d_out_p, s, st));
     if (c->timed) EF_CK(cudaEventRecord(c->ev1, s));
     c->stats.dominant_kernel_launches = 1 + c->nblocks;
+    // the sums over patterns and bitstrings, one array after the other, in one copy
     std::vector<std::vector<cd>> tbar(c->nblocks), sbar(c->nblocks), ebar(c->nblocks);
     std::vector<cd> pbar;
+    ef::SumJobs jobs{};
+    std::vector<std::vector<cd>*> to;
+    auto job = [&](const DBuf& in, int64_t count, int64_t width, std::vector<cd>& out) {
+        out.resize(width);
+        to.push_back(&out);
+        jobs.job[jobs.n++] = {in.as<double2>(), nullptr, count, width};
+    };
     for (int b = 0; b < c->nblocks; ++b) {
         HostBlock& B = c->blk[b];
         const int64_t ny = (int64_t)1 << B.r;
-        const int64_t wT = (int64_t)B.L * B.n * B.n, wS = (int64_t)B.n * B.eta, wE = (int64_t)1 << B.r_loc;
-        EF_CK(ef::launch_sum_rows(B.dTbar.as<double2>(), ny, wT, wT, B.dSumT.as<double2>(), s, st));
-        EF_CK(ef::launch_sum_rows(B.dSbar.as<double2>(), ny, wS, wS, B.dSumS.as<double2>(), s, st));
-        EF_CK(ef::launch_sum_rows(B.dEbar.as<double2>(), nb, wE, wE, B.dSumE.as<double2>(), s, st));
-        tbar[b].resize(wT);
-        sbar[b].resize(wS);
-        ebar[b].resize(wE);
-        if (wT) EF_CK(cudaMemcpyAsync(tbar[b].data(), B.dSumT.p, wT * sizeof(double2), cudaMemcpyDeviceToHost, s));
-        EF_CK(cudaMemcpyAsync(sbar[b].data(), B.dSumS.p, wS * sizeof(double2), cudaMemcpyDeviceToHost, s));
-        EF_CK(cudaMemcpyAsync(ebar[b].data(), B.dSumE.p, wE * sizeof(double2), cudaMemcpyDeviceToHost, s));
+        job(B.dTbar, ny, (int64_t)B.L * B.n * B.n, tbar[b]);
+        job(B.dSbar, ny, (int64_t)B.n * B.eta, sbar[b]);
+        job(B.dEbar, nb, (int64_t)1 << B.r_loc, ebar[b]);
     }
-    if (c->nblocks == 2) {
-        const int64_t wP = (int64_t)1 << ksh;
-        EF_CK(ef::launch_sum_rows(c->dPbar.as<double2>(), nb, wP, wP, c->dSumP.as<double2>(), s, st));
-        pbar.resize(wP);
-        EF_CK(cudaMemcpyAsync(pbar.data(), c->dSumP.p, wP * sizeof(double2), cudaMemcpyDeviceToHost, s));
+    if (c->nblocks == 2) job(c->dPbar, nb, (int64_t)1 << ksh, pbar);
+    int64_t values = 0;
+    for (int i = 0; i < jobs.n; ++i) values += jobs.job[i].width;
+    EF_CK(c->dSums.ensure(std::max<int64_t>(values, 1) * sizeof(double2)));
+    double2* at = c->dSums.as<double2>();
+    for (int i = 0; i < jobs.n; ++i) {
+        jobs.job[i].out = at;
+        at += jobs.job[i].width;
     }
+    EF_CK(ef::launch_sum_rows(jobs, s, st));
+    std::vector<cd> sums(values);
+    if (values) EF_CK(cudaMemcpyAsync(sums.data(), c->dSums.p, values * sizeof(double2), cudaMemcpyDeviceToHost, s));
     EF_CK(cudaStreamSynchronize(s));
+    {
+        const cd* from = sums.data();
+        for (std::vector<cd>* v : to) {
+            std::copy(from, from + v->size(), v->begin());
+            from += v->size();
+        }
+    }
     c->stats.kernel_launches = st.launches;
     c->stats.executed_minor_lus = 2 * st.executed_lus;
     grad_finish(c, tbar, sbar, ebar, pbar, grad);

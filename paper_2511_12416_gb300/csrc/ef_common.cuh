@@ -66,6 +66,14 @@ __device__ __forceinline__ double recip(double m) { return 1.0 / m; }
 // such pivots when rounding noise stands where an exact zero belongs.
 __device__ __forceinline__ float min_pivot2(float) { return 1.17549435e-38f; }
 __device__ __forceinline__ double min_pivot2(double) { return 2.2250738585072014e-308; }
+// Pivot key of an FP64 entry: the leading 32 bits of its larger component, which
+// order as integers (the pivot is within a factor sqrt(2) of the largest).
+// Comparing |a|^2 takes the FP64 pipe three instructions an entry, 64 cycles a
+// warp each. For well-conditioned matrices only: where a minor is singular up
+// to rounding its value hangs on the pivots, and the Exact minors keep |a|^2.
+__device__ __forceinline__ int pivot_key(double2 a) {
+    return max(__double2hiint(a.x) & 0x7fffffff, __double2hiint(a.y) & 0x7fffffff);
+}
 // 1/u^2 for the unit roundoff u of the type (2^-24, 2^-53)
 __device__ __forceinline__ float inv_u2(float) { return 281474976710656.0f; }
 __device__ __forceinline__ double inv_u2(double) { return 81129638414606681695789005144064.0; }

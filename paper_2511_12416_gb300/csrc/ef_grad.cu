@@ -300,6 +300,7 @@ __global__ void __launch_bounds__(128) k_grad_minors(GradDev G, int blk, const u
     double2* xb = xs + (size_t)(L + 1) * ne;           // [n][ETA] running Xbar
     uint64_t* rmask = reinterpret_cast<uint64_t*>(xb + ne);  // [NT] local row masks
     int* sgn = reinterpret_cast<int*>(rmask + NT);     // [n]
+    unsigned* occ = reinterpret_cast<unsigned*>(sgn + n);  // [n][NT / 32]
     const int tid = threadIdx.x;
     const uint32_t z = blockIdx.x;
     const double2* Mz = B.M64 + (size_t)z * ne;
@@ -334,23 +335,27 @@ __global__ void __launch_bounds__(128) k_grad_minors(GradDev G, int blk, const u
             }
         }
         rmask[tid] = ok ? lm : 0ull;
-        if (!ok)
-            for (int e = 0; e < ETA * ETA; ++e) gt[e] = make_double2(0.0, 0.0);
+        // who of the tile occupies mode m: a word per warp
+        for (int m = 0; m < n; ++m) {
+            const unsigned who = __ballot_sync(0xffffffffu, ok && ((lm >> m) & 1ull));
+            if ((tid & 31) == 0) occ[m * (NT / 32) + (tid >> 5)] = who;
+        }
         __syncthreads();
-        // fixed-order accumulation: element (m, j) sums the tile's threads in order
+        // fixed-order accumulation: element (m, j) sums the tile's threads that occupy m, in order
+        // (asking every thread of the tile took the FP64 pipe 1024 instructions a tile instead
+        // of 360: a warp adds for all its lanes' modes)
         for (int e = tid; e < ne; e += NT) {
             const int m = e / ETA, j = e - m * ETA;
             double2 acc = ubar[e];
             const uint64_t below = (m == 63) ? ~0ull >> 1 : ((1ull << m) - 1ull);
-            for (int t = 0; t < NT; ++t) {
-                const uint64_t msk = rmask[t];
-                if ((msk >> m) & 1ull) {
-                    const int i = __popcll(msk & below);
+            for (int w = 0; w < NT / 32; ++w)
+                for (unsigned who = occ[m * (NT / 32) + w]; who; who &= who - 1) {
+                    const int t = 32 * w + __ffs(who) - 1;
+                    const int i = __popcll(rmask[t] & below);
                     const double2 g = gs[(size_t)t * GS + i * ETA + j];
                     acc.x += g.x;
                     acc.y += g.y;
                 }
-            }
             ubar[e] = acc;
         }
         __syncthreads();
@@ -421,9 +426,9 @@ __global__ void __launch_bounds__(128) k_grad_minors(GradDev G, int blk, const u
 
 size_t grad_minors_smem(int n, int eta, int L) {
     const size_t ne = (size_t)n * eta;
-    // matches k_grad_minors: [128][(eta^2) | 1] cotangent blocks, ubar, X_0..X_L, Xbar, row masks, signs
+    // matches k_grad_minors: [128][(eta^2) | 1] cotangent blocks, ubar, X_0..X_L, Xbar, row masks, signs, occupations
     return (size_t)128 * ((eta * eta) | 1) * sizeof(double2) + ne * sizeof(double2) * (3 + L) +
-           128 * sizeof(uint64_t) + (size_t)n * sizeof(int);
+           128 * sizeof(uint64_t) + (size_t)n * 5 * sizeof(int);
 }
 
 template <int ETA>
@@ -467,41 +472,56 @@ cudaError_t launch_grad(const GradDev& g, const uint64_t* bits, int64_t nb, cons
 }
 
 // ---------------------------------------------------------------- fixed-order sums
-// out[e] = sum_{k < count} in[k * stride + e] for e < width (complex), k ascending.
-// out[e] = sum_k in[k * stride + e] for e < width, in a fixed order: a CTA
-// covers 32 consecutive e (one per lane); warp w adds rows w, w + 32, w + 64,
-// ... and warp 0 then adds the 32 warps' partial sums in order. Splitting the
-// count over 32 warps keeps the chains of dependent FP64 additions short.
-__global__ void __launch_bounds__(1024) k_sum_rows(const double2* __restrict__ in, int64_t count, int64_t stride,
-                                                   int64_t width, double2* __restrict__ out) {
+// out[e] = sum_k in[k * width + e] for e < width, in a fixed order, for several
+// arrays in one launch (blockIdx.y): a CTA covers 32 consecutive e (one per lane);
+// warp w adds rows w, w + 32, w + 64, ... and warp 0 then adds the 32 warps'
+// partial sums in order. Splitting the count over 32 warps keeps the chains of
+// dependent FP64 additions short, eight loads ahead hide the memory's latency, and
+// one launch runs the narrow arrays (one or a few CTAs each, 82 us in launches of
+// their own at 4096 rows) side by side.
+__global__ void __launch_bounds__(1024) k_sum_rows(const __grid_constant__ SumJobs jobs) {
     __shared__ double2 part[32][33];
+    const SumJobs::Job J = jobs.job[blockIdx.y];
+    if ((int64_t)blockIdx.x * 32 >= J.width) return;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int64_t e = (int64_t)blockIdx.x * 32 + lane;
     double ax = 0.0, ay = 0.0;
-    if (e < width)
-        for (int64_t k = w; k < count; k += 32) {
-            const double2 v = in[k * stride + e];
+    if (e < J.width) {
+        int64_t k = w;
+        for (; k + 7 * 32 < J.count; k += 8 * 32) {
+            double2 v[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) v[q] = J.in[(k + 32 * q) * J.width + e];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                ax += v[q].x;
+                ay += v[q].y;
+            }
+        }
+        for (; k < J.count; k += 32) {
+            const double2 v = J.in[k * J.width + e];
             ax += v.x;
             ay += v.y;
         }
+    }
     part[w][lane] = make_double2(ax, ay);
     __syncthreads();
-    if (w == 0 && e < width) {
+    if (w == 0 && e < J.width) {
         double sx = 0.0, sy = 0.0;
         for (int q = 0; q < 32; ++q) {
             sx += part[q][lane].x;
             sy += part[q][lane].y;
         }
-        out[e] = make_double2(sx, sy);
+        J.out[e] = make_double2(sx, sy);
     }
 }
 
-cudaError_t launch_sum_rows(const double2* in, int64_t count, int64_t stride, int64_t width, double2* out,
-                            cudaStream_t s, LaunchStats& st) {
-    if (width <= 0) return cudaSuccess;
-    const int64_t blocks = (width + 31) / 32;
+cudaError_t launch_sum_rows(const SumJobs& jobs, cudaStream_t s, LaunchStats& st) {
+    int64_t blocks = 0;
+    for (int i = 0; i < jobs.n; ++i) blocks = std::max(blocks, (jobs.job[i].width + 31) / 32);
+    if (blocks <= 0) return cudaSuccess;
     if (blocks > 2147483647ll) return cudaErrorInvalidValue;
-    k_sum_rows<<<(unsigned)blocks, 1024, 0, s>>>(in, count, stride, width, out);
+    k_sum_rows<<<dim3((unsigned)blocks, (unsigned)jobs.n), 1024, 0, s>>>(jobs);
     st.launches += 1;
     return cudaGetLastError();
 }

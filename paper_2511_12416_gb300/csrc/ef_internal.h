@@ -292,8 +292,16 @@ cudaError_t launch_exact_combine(const ExactCombineDev& c, const uint64_t* bits,
 cudaError_t launch_grad(const GradDev& g, const uint64_t* bits, int64_t nb, const double* grad_p,
                         double* out_p, cudaStream_t s, LaunchStats& st);
 size_t grad_minors_smem(int n, int eta, int L);
-cudaError_t launch_sum_rows(const double2* in, int64_t count, int64_t stride, int64_t width, double2* out,
-                            cudaStream_t s, LaunchStats& st);
+// fixed-order sums over the rows of several arrays (count rows of width values each)
+struct SumJobs {
+    struct Job {
+        const double2* in;
+        double2* out;
+        int64_t count, width;
+    } job[3 * kMaxBlocks + 1];
+    int n;
+};
+cudaError_t launch_sum_rows(const SumJobs& jobs, cudaStream_t s, LaunchStats& st);
 // Raw Estimate: K form or not and the bytes of a bitstring's image; bytes of
 // the samples of one item; the launch over the items
 // (all bitstrings, or a.list); the per-bitstring finalisation (listed: the
