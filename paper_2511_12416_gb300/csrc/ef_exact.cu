@@ -219,7 +219,7 @@ cudaError_t launch_dedup(const ExactBlockDev& b0, const ExactBlockDev& b1, const
 
 struct NoDedup {};
 template <typename D>  // DedupDev (two mode blocks: blockIdx.y = 2 searches) or NoDedup
-__global__ void __launch_bounds__(128) k_build_branches(ExactBlockDev B0, ExactBlockDev B1, int want32, int* count,
+__global__ void __launch_bounds__(512) k_build_branches(ExactBlockDev B0, ExactBlockDev B1, int want32, int* count,
                                                         unsigned long long* recomp, D dedup) {
     cudaGridDependencySynchronize();  // see launch_pdl
     extern __shared__ double2 smb[];
@@ -324,25 +324,30 @@ cudaError_t launch_build_branches(const ExactBlockDev& b0, const ExactBlockDev& 
     if (nblk < 1 || nblk > 2) return cudaErrorInvalidValue;
     size_t smem = 0;
     uint32_t ny = 1;
+    int entries = 1;
     for (int i = 0; i < nblk; ++i) {
         const ExactBlockDev& b = i ? b1 : b0;
         smem = std::max(smem, (size_t)2 * b.n * b.eta * sizeof(double2) + (size_t)b.n * sizeof(int));
         if (want32 && b.n <= kBuildFFModes)  // float-pair path: the layer's T staged as float pairs too
             smem = std::max(smem, (size_t)(2 * b.n * b.eta + b.n * b.n) * sizeof(float4) + (size_t)b.n * sizeof(int));
         ny = std::max(ny, 1u << b.r);
+        entries = std::max(entries, b.n * b.eta);
     }
     const ExactBlockDev& bb = nblk == 2 ? b1 : b0;
+    // a thread per entry of a pattern's n x eta matrix up to 512: each adds n float-pair products a
+    // layer, a latency chain (24 modes, 12 particles, 5 layers: 55 us with 128 threads)
     const unsigned gx = std::min<uint32_t>(ny, (uint32_t)sm_count() * 16u);
+    const unsigned nt = (unsigned)std::min(512, std::max(128, (entries + 31) / 32 * 32));
     cudaError_t e;
     st.launches += 1;
     if (dedup) {
         if (nblk != 2) return cudaErrorInvalidValue;
         if ((e = raise_dynamic_smem((const void*)k_build_branches<DedupDev>, smem)) != cudaSuccess) return e;
-        return launch_pdl(k_build_branches<DedupDev>, dim3(gx, 3u), dim3(128), smem, s, b0, bb, want32 ? 1 : 0, count, recomp,
+        return launch_pdl(k_build_branches<DedupDev>, dim3(gx, 3u), dim3(nt), smem, s, b0, bb, want32 ? 1 : 0, count, recomp,
                           *dedup);
     }
     if ((e = raise_dynamic_smem((const void*)k_build_branches<NoDedup>, smem)) != cudaSuccess) return e;
-    return launch_pdl(k_build_branches<NoDedup>, dim3(gx, (unsigned)nblk), dim3(128), smem, s, b0, bb, want32 ? 1 : 0, count,
+    return launch_pdl(k_build_branches<NoDedup>, dim3(gx, (unsigned)nblk), dim3(nt), smem, s, b0, bb, want32 ? 1 : 0, count,
                       recomp, NoDedup{});
 }
 
