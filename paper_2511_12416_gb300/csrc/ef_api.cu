@@ -189,6 +189,7 @@ struct ef_circuit {
     DBuf dWS, dWS32, dWSFF, dList, dListCount, dRecomp, dDedup, dMarks, dBits, dOut, dErr, dGradP, dGrad, dPbar, dSums;
     DBuf daT, daq, daq32, dalayer, damodes, dagpair, daPart, dCounters, daList, daSamples, daImage;
     cudaStream_t own_stream = nullptr;
+    ef::SideStream side;  // a second slab of a Raw Estimate call
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     bool timed = false;
     cudaStream_t last_stream = nullptr;
@@ -217,6 +218,9 @@ struct ef_circuit {
         if (ev0) cudaEventDestroy(ev0);
         if (ev1) cudaEventDestroy(ev1);
         if (own_stream) cudaStreamDestroy(own_stream);
+        if (side.fork) cudaEventDestroy(side.fork);
+        if (side.join) cudaEventDestroy(side.join);
+        if (side.stream) cudaStreamDestroy(side.stream);
     }
 };
 
@@ -1657,7 +1661,8 @@ int approx_setup(ef_circuit* c, int64_t nb, int64_t t, uint64_t seed, uint64_t b
     }
     // Workspace of a slab of items: samples (K form) and the bitstrings' images, for
     // the FP32 pass and the FP64 redo alike, within 512 MiB (a slab of the 52-qubit
-    // LUCJ circuit is 880 bitstrings: several waves of the evaluation).
+    // LUCJ circuit is 800 bitstrings: several waves of the evaluation); two of them
+    // where a call has more items than a slab.
     a.n_seg = (int)ef::approx_segments(a.traj_per_cta);
     a.id_bits = a.k <= 256 ? 8 : 16;
     {
@@ -1681,9 +1686,31 @@ int approx_setup(ef_circuit* c, int64_t nb, int64_t t, uint64_t seed, uint64_t b
     int64_t slab = bytes <= budget ? std::min<int64_t>(budget / bytes, 1 << 20) * a.n_chunks
                                    : std::max<int64_t>(1, (budget - img) / std::max<int64_t>(item, 1));
     slab = std::min(std::min(slab, items), std::max<int64_t>(1, 2147483647ll / a.n_seg));
+    // several slabs in flight are worth it from about two waves of the evaluation's CTAs each and
+    // some milliseconds of sampling (10^9 Philox blocks)
+    const int64_t wave = 2 * sms;
+    if (items >= 4 * wave && slab > (items + 3) / 4 && bytes <= budget && (double)nb * t * ((a.k + 3) / 4) >= 1e9) {
+        slab = (std::max<int64_t>(2 * wave, (items + 3) / 4) + a.n_chunks - 1) / a.n_chunks * a.n_chunks;
+        slab = std::min(slab, items);
+    }
     a.slab_items = slab;
-    EF_CK(c->daSamples.ensure(item ? ef::approx_sample_bytes(a, slab, &o_ent, &o_sum, &o_cnt) : 0));
-    EF_CK(c->daImage.ensure((size_t)std::min<int64_t>(std::max<int64_t>(nb, 1), slab / a.n_chunks + 2) * img));
+    const bool two = items > slab;
+    const size_t samples = item ? (ef::approx_sample_bytes(a, slab, &o_ent, &o_sum, &o_cnt) + 255) / 256 * 256 : 0;
+    const size_t images = ((size_t)std::min<int64_t>(std::max<int64_t>(nb, 1), slab / a.n_chunks + 2) * img + 255) / 256 * 256;
+    EF_CK(c->daSamples.ensure((two ? 2 : 1) * samples));
+    EF_CK(c->daImage.ensure((two ? 2 : 1) * images));
+    if (two) {
+        if (!c->side.stream) {
+            EF_CK(cudaStreamCreateWithFlags(&c->side.stream, cudaStreamNonBlocking));
+            EF_CK(cudaEventCreateWithFlags(&c->side.fork, cudaEventDisableTiming));
+            EF_CK(cudaEventCreateWithFlags(&c->side.join, cudaEventDisableTiming));
+        }
+        a.alt_samples = (int64_t)samples;
+        a.alt_img = (int64_t)images;
+        int least = 0, greatest = 0;
+        EF_CK(cudaDeviceGetStreamPriorityRange(&least, &greatest));
+        a.eval_priority = greatest;
+    }
     unsigned char* sp = c->daSamples.as<unsigned char>();
     if (item) {
         a.codes = reinterpret_cast<uint16_t*>(sp);
@@ -1708,7 +1735,7 @@ int approx_enqueue(ef_circuit* c, const ef::ApproxDev& a, const uint64_t* d_bits
     EF_CK(cudaMemsetAsync(a.counters, 0, 8 * sizeof(unsigned long long), s));
     EF_CK(cudaMemsetAsync(list_count, 0, sizeof(int), s));
     if (c->timed) EF_CK(cudaEventRecord(c->ev0, s));
-    EF_CK(ef::launch_approx(a, d_bits, fp64, s, st));
+    EF_CK(ef::launch_approx(a, d_bits, fp64, c->side, s, st));
     if (c->timed) EF_CK(cudaEventRecord(c->ev1, s));
     EF_CK(ef::launch_approx_finalize(a, d_out, d_se, d_err, autofix ? list : nullptr, list_count, false, s, st));
     if (autofix) {
@@ -1716,7 +1743,7 @@ int approx_enqueue(ef_circuit* c, const ef::ApproxDev& a, const uint64_t* d_bits
         r.list = list;
         r.list_count = list_count;
         r.counters = a.counters + 4;  // the redo's own flips, LUs and rank-one minors
-        EF_CK(ef::launch_approx(r, d_bits, true, s, st));
+        EF_CK(ef::launch_approx(r, d_bits, true, c->side, s, st));
         EF_CK(ef::launch_approx_finalize(r, d_out, d_se, d_err, nullptr, nullptr, true, s, st));
     }
     return EF_OK;

@@ -181,6 +181,8 @@ struct ApproxDev {
     float* hsums;            // FP32: eight sums per thread over the small trajectories of an item
     unsigned char* img;      // per bitstring of a slab: what the set-up leaves for the evaluation
     int64_t img_bytes;
+    int64_t alt_samples, alt_img;  // byte offsets of a second slab's samples and images (0: none)
+    int eval_priority;       // launch priority of the evaluation when two slabs are in flight
     int kform;               // 1: trajectory minors through K (every block has <= 64 flippable pairs)
     double kappa_max;        // A0 with ||A0||_1 ||A0^-1||_1 above this takes the rank-one form
     double err_coef;         // FP32 error estimate: K u32 (0: no estimate)
@@ -241,19 +243,26 @@ cudaError_t raise_dynamic_smem(const void* kernel, size_t bytes);
 // (and writes nothing the previous kernel reads) exactly as with an ordinary
 // launch.
 template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
-                       Args&&... args) {
+cudaError_t launch_pdl_at(int priority, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                          Args&&... args) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributePriority;
+    attr[1].val.priority = priority;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = priority ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                       Args&&... args) {
+    return launch_pdl_at(0, kernel, grid, block, smem, s, static_cast<Args&&>(args)...);
 }
 
 // branch matrices of nblk (1 or 2) mode blocks in one launch, which also clears
@@ -311,7 +320,13 @@ size_t approx_sample_bytes(const ApproxDev& a, int64_t items, size_t* entries, s
 int64_t approx_segments(int64_t traj_per_cta);  // segments of an item's stream
 int approx_segment_traj();                      // trajectories of a segment
 int approx_eta_template(const ApproxDev& a);
-cudaError_t launch_approx(const ApproxDev& a, const uint64_t* bits, bool fp64, cudaStream_t s, LaunchStats& st);
+// A stream and events for a second slab in flight.
+struct SideStream {
+    cudaStream_t stream = nullptr;
+    cudaEvent_t fork = nullptr, join = nullptr;
+};
+cudaError_t launch_approx(const ApproxDev& a, const uint64_t* bits, bool fp64, const SideStream& side, cudaStream_t s,
+                          LaunchStats& st);
 cudaError_t launch_approx_finalize(const ApproxDev& a, double* out, double* stderr_out, double* err_out,
                                    int* append_list, int* append_count, bool listed, cudaStream_t s,
                                    LaunchStats& st);
