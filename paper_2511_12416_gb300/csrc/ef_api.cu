@@ -186,7 +186,7 @@ struct ef_circuit {
     double R0 = 1.0;
 
     bool dirty = true;
-    DBuf dWS, dWS32, dWSFF, dList, dListCount, dRecomp, dDedup, dMarks, dBits, dOut, dErr, dGradP, dGrad, dPbar, dSums;
+    DBuf dWS, dWS32, dWSFF, dList, dListCount, dRecomp, dDedup, dBits, dOut, dErr, dGradP, dGrad, dPbar, dSums;
     DBuf daT, daq, daq32, dalayer, damodes, dagpair, daPart, dCounters, daList, daSamples, daImage;
     cudaStream_t own_stream = nullptr;
     ef::SideStream side;  // a second slab of a Raw Estimate call
@@ -206,7 +206,7 @@ struct ef_circuit {
 
     template <typename F> void for_each_buf(F f) {
         for (int b = 0; b < ef::kMaxBlocks; ++b) blk[b].for_each_buf(f);
-        for (DBuf* d : {&dWS, &dWS32, &dWSFF, &dList, &dListCount, &dRecomp, &dDedup, &dMarks, &dBits, &dOut, &dErr, &dGradP, &dGrad, &dPbar, &dSums, &daT,
+        for (DBuf* d : {&dWS, &dWS32, &dWSFF, &dList, &dListCount, &dRecomp, &dDedup, &dBits, &dOut, &dErr, &dGradP, &dGrad, &dPbar, &dSums, &daT,
                         &daq, &daq32, &dalayer, &damodes, &dagpair, &daPart, &dCounters, &daList, &daSamples, &daImage})
             f(*d);
     }
@@ -1227,7 +1227,10 @@ int exact_buffers(ef_circuit* c, int64_t cap, bool dedup, ExactBuffers& eb) {
         uint32_t h = 1;
         while ((int64_t)h < 2 * cap) h <<= 1;
         d.hmask = h - 1;
-        EF_CK(c->dDedup.ensure(((size_t)2 * h + 4 + 4 * (size_t)cap) * sizeof(int) + (size_t)cap * 4 * sizeof(uint64_t)));
+        if (per_minor_recompute(c))
+            eb.mark_words = (int)((((int64_t)1 << c->blk[0].r) + ((int64_t)1 << c->blk[1].r) + 31) / 32);
+        EF_CK(c->dDedup.ensure(((size_t)2 * h + 4 + (4 + (size_t)eb.mark_words) * (size_t)cap) * sizeof(int) +
+                               (size_t)cap * 4 * sizeof(uint64_t)));
         d.ubits[0] = c->dDedup.as<uint64_t>();
         d.ubits[1] = d.ubits[0] + 2 * cap;
         int* at = reinterpret_cast<int*>(d.ubits[1] + 2 * cap);
@@ -1244,11 +1247,7 @@ int exact_buffers(ef_circuit* c, int64_t cap, bool dedup, ExactBuffers& eb) {
             eb.blk[b].rep = d.rep[b];
             eb.blk[b].ucol = d.ucol[b];
         }
-        if (per_minor_recompute(c)) {
-            eb.mark_words = (int)((((int64_t)1 << c->blk[0].r) + ((int64_t)1 << c->blk[1].r) + 31) / 32);
-            EF_CK(c->dMarks.ensure((size_t)cap * eb.mark_words * sizeof(uint32_t)));
-            eb.marks = c->dMarks.as<uint32_t>();
-        }
+        eb.marks = reinterpret_cast<uint32_t*>(at + 4 * (size_t)cap);
     }
     eb.list = c->dList.as<int>();
     eb.list2 = eb.list + cap;
