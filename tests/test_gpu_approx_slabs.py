@@ -53,6 +53,23 @@ def test_slabs_in_a_batch_graph(lib):
             lib.ef_batch_destroy(b)
 
 
+@pytest.mark.parametrize("prec,nb,t", [("fp64", 1900, 100_000), ("auto", 1900, 100_000), ("auto", 1825, 250_001)])
+def test_long_items_are_cut(lib, prec, nb, t):
+    # large angles: most trajectories flip several gates, so one bitstring's samples pass 1 MB and its item is
+    # cut; the small calls split their few bitstrings finely instead. The trajectories are the same, the sums are
+    # grouped differently: FP64 within 10^5 roundings of the extent (100), FP32 within twice tol
+    c = W.lucj_circuit(6, 3, 3, 1, n_onsite=6, n_same=3, angle_sampler=W.normal_var(1.0), seed=11)
+    bits = W.spin_sector_bitstrings(6, 3, 3, nb, np.random.default_rng(5))
+    with lib.Circuit(c.n_modes, c.occupation, c.gates,
+                     precision=lib.EF_PREC_FP64 if prec == "fp64" else lib.EF_PREC_AUTO) as h:
+        p, se = lib.ef_prob_approx(h.handle, bits, t, seed=3)
+        assert np.array_equal(lib.ef_prob_approx(h.handle, bits, t, seed=3)[0], p)
+        for lo, hi in ((0, 30), (nb - 7, nb)):
+            q, sq = lib.ef_prob_approx(h.handle, bits[lo:hi], t, seed=3, index_base=lo)
+            assert np.allclose(p[lo:hi], q, rtol=1e-9 if prec == "fp64" else 2e-5, atol=1e-9 if prec == "fp64" else 1e-12)
+            assert np.allclose(se[lo:hi], sq, rtol=1e-6 if prec == "fp64" else 1e-3, atol=1e-9)
+
+
 def test_no_particles(lib):
     recs = [(W.GIVENS, 0, 1, 0.3, 0.1), (W.CPHASE, 0, 2, 0.9, 0.0), (W.CPHASE, 1, 3, -1.2, 0.0), (W.GIVENS, 2, 3, 0.7, 0.2)]
     c = W.Circuit(4, np.zeros(2, dtype=np.uint64), W.make_gates(recs))
