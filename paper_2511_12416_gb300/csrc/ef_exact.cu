@@ -733,7 +733,8 @@ __device__ __forceinline__ float err_term(const ExactCombineDev& C, int B, size_
     const uint16_t code = C.E32[B][idx];
     return C.src == 2 && redone(C, B, b, z, code) ? 0.f : err_term_value(code);
 }
-// Listing a bitstring's determinants: clear its marks, then set those of the listed ones.
+// Listing a flagged bitstring's determinants (every one has a budget of 0 or more): clear its
+// marks, which the re-estimate reads, then set those of the listed ones.
 __device__ __forceinline__ void clear_marks(const ExactCombineDev& C, int64_t b, int tid, int nt) {
     if (C.rep[0])
         for (int i = tid; i < C.mark_words; i += nt) C.marks[b * C.mark_words + i] = 0u;
@@ -1034,7 +1035,7 @@ __global__ void __launch_bounds__(256, 3) k_exact_combine(ExactCombineDev C, con
             } else if (err) {
                 err[b] = e;
             }
-            const bool flag = append_list && e > C.tol;
+            const bool flag = append_list && !(e <= C.tol);
             if (flag) {
                 const int idx = atomicAdd(append_count, 1);
                 append_list[idx] = (int)b;
@@ -1046,7 +1047,7 @@ __global__ void __launch_bounds__(256, 3) k_exact_combine(ExactCombineDev C, con
                 // cannot sum past half of it
                 const double st = C.tol * fmax(p, C.p_floor) / (sp + sqrt(fma(C.tol, fmax(p, C.p_floor), p)));
                 const double vt = st / C.err_coef;
-                s_theta = flag ? 0.5 * vt * vt / (double)C.minors : -1.0;
+                s_theta = !flag ? -1.0 : vt >= 0.0 ? 0.5 * vt * vt / (double)C.minors : 0.0;
             }
         }
         if (emit) {
@@ -1058,7 +1059,7 @@ __global__ void __launch_bounds__(256, 3) k_exact_combine(ExactCombineDev C, con
                 for (int B = 0; B < C.nblocks; ++B) {
                     const int nz = 1 << C.r[B];
                     for (int z = tid; z < nz; z += NT)
-                        if ((double)smV[B * voff1 + z] > theta) list_minor(C, B, b, z);
+                        if (!((double)smV[B * voff1 + z] <= theta)) list_minor(C, B, b, z);
                 }
             }
         }
@@ -1241,9 +1242,10 @@ __global__ void __launch_bounds__(NT, 3) k_exact_combine_ffr(ExactCombineDev C, 
                 append_list[atomicAdd(append_count, 1)] = (int)b;
                 if (emit) {
                     // half the variance at which the estimate equals tol
+                    // (0 / 0 where p is zero and tol max(p, floor) underflows: nothing may be left)
                     const float st = tol * pm / (sp + sqrtf(fmaf(tol, pm, pf)));
                     const float vt = st / ec;
-                    budget = 0.5f * vt * vt;
+                    budget = vt >= 0.f ? 0.5f * vt * vt : 0.f;
                 }
             }
         }
@@ -1497,9 +1499,11 @@ __global__ void __launch_bounds__(128, (RL >= 5 ? 2 : 3)) k_exact_combine_wp(Exa
             if (append_list && !(e <= tol)) {
                 append_list[atomicAdd(append_count, 1)] = (int)b;
                 if (emit) {
+                    // half the variance at which the estimate equals tol; 0 / 0 where p is zero and
+                    // tol max(p, floor) underflows: nothing may be left
                     const float st = tol * pm / (sp + sqrtf(fmaf(tol, pm, pf)));
                     const float vt = st / ec;
-                    budget = 0.5f * vt * vt;  // half the variance at which the estimate equals tol
+                    budget = vt >= 0.f ? 0.5f * vt * vt : 0.f;
                 }
             }
         }
