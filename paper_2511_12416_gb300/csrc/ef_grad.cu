@@ -300,7 +300,9 @@ __global__ void __launch_bounds__(128) k_grad_minors(GradDev G, int blk, const u
     double2* xb = xs + (size_t)(L + 1) * ne;           // [n][ETA] running Xbar
     uint64_t* rmask = reinterpret_cast<uint64_t*>(xb + ne);  // [NT] local row masks
     int* sgn = reinterpret_cast<int*>(rmask + NT);     // [n]
-    unsigned* occ = reinterpret_cast<unsigned*>(sgn + n);  // [n][NT / 32]
+    // [n][NT / 32] who of a tile occupies a mode: in the place of X_0, which is written after the tiles
+    unsigned* occ = reinterpret_cast<unsigned*>(xs);
+    static_assert(NT / 32 * sizeof(unsigned) <= ETA * sizeof(double2), "occupations fit X_0");
     const int tid = threadIdx.x;
     const uint32_t z = blockIdx.x;
     const double2* Mz = B.M64 + (size_t)z * ne;
@@ -426,9 +428,9 @@ __global__ void __launch_bounds__(128) k_grad_minors(GradDev G, int blk, const u
 
 size_t grad_minors_smem(int n, int eta, int L) {
     const size_t ne = (size_t)n * eta;
-    // matches k_grad_minors: [128][(eta^2) | 1] cotangent blocks, ubar, X_0..X_L, Xbar, row masks, signs, occupations
+    // matches k_grad_minors: [128][(eta^2) | 1] cotangent blocks, ubar, X_0..X_L, Xbar, row masks, signs
     return (size_t)128 * ((eta * eta) | 1) * sizeof(double2) + ne * sizeof(double2) * (3 + L) +
-           128 * sizeof(uint64_t) + (size_t)n * 5 * sizeof(int);
+           128 * sizeof(uint64_t) + (size_t)n * sizeof(int);
 }
 
 template <int ETA>
