@@ -1,0 +1,54 @@
+"""Order of a call's slabs on two streams (csrc/ef_slabs.h), compiled with the host compiler."""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2511_12416_gb300", "csrc")
+
+MAIN = r"""
+#include <cstdio>
+#include <cstdlib>
+#include "ef_slabs.h"
+int main(int argc, char** argv) {
+    const long items = atol(argv[1]), slab = atol(argv[2]), two = atol(argv[3]), bad = atol(argv[4]);
+    long n = 0;
+    const auto step = [&](const char* what) {
+        printf("%s ", what);
+        return (int)(bad == ++n ? 100 + n : 0);
+    };
+    const int e = ef::for_slabs<int>(items, slab, two, [&] { return step("fork"); }, [&] { return step("join"); },
+        [&](int64_t i0, int64_t k, int turn) {
+            printf("%ld+%ld@%d ", (long)i0, (long)k, turn);
+            return bad == ++n ? (int)(100 + n) : 0;
+        });
+    printf("%d\n", e);
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def run(tmp_path_factory):
+    cxx = shutil.which("g++")
+    if cxx is None:
+        pytest.skip("no host compiler")
+    d = tmp_path_factory.mktemp("slabs")
+    (d / "m.cpp").write_text(MAIN)
+    subprocess.run([cxx, "-std=c++17", "-I", CSRC, str(d / "m.cpp"), "-o", str(d / "m")], check=True)
+    return lambda *a: subprocess.run([str(d / "m"), *map(str, a)], check=True, capture_output=True, text=True).stdout.split()
+
+
+def test_slabs_cover_the_items_in_turn(run):
+    assert run(7, 3, 0, 0) == ["0+3@0", "3+3@0", "6+1@0", "0"]
+    assert run(7, 3, 1, 0) == ["fork", "0+3@0", "3+3@1", "6+1@0", "join", "0"]
+    assert run(3, 3, 0, 0) == ["0+3@0", "0"]
+
+
+def test_a_failed_launch_still_joins(run):
+    # steps: fork 1, launches 2 .., join last
+    assert run(9, 3, 1, 3) == ["fork", "0+3@0", "3+3@1", "join", "103"]
+    assert run(9, 3, 1, 2) == ["fork", "0+3@0", "join", "102"]
+    assert run(9, 3, 1, 5) == ["fork", "0+3@0", "3+3@1", "6+3@0", "join", "105"]
+    assert run(9, 3, 1, 1) == ["fork", "101"]  # nothing is on the side stream yet
+    assert run(9, 3, 0, 2) == ["0+3@0", "3+3@0", "102"]
