@@ -25,6 +25,7 @@
 #include <vector>
 
 #include "ef_internal.h"
+#include "ef_slabs.h"
 #include "extraferm.h"
 
 using cd = std::complex<double>;
@@ -1695,22 +1696,11 @@ int approx_setup(ef_circuit* c, int64_t nb, int64_t t, uint64_t seed, uint64_t b
     const int64_t img = std::max(first.img_bytes, redo.img_bytes);
     size_t o_ent, o_sum, o_cnt;
     const int64_t item = first.kform || redo.kform ? (int64_t)ef::approx_sample_bytes(a, 1, &o_ent, &o_sum, &o_cnt) : 0;
-    const int64_t budget = slab_bytes, bytes = img + item * a.n_chunks;
-    const int64_t items = std::max<int64_t>(nb, 1) * a.n_chunks;
-    int64_t slab = bytes <= budget ? std::min<int64_t>(budget / bytes, 1 << 20) * a.n_chunks
-                                   : std::max<int64_t>(1, (budget - img) / std::max<int64_t>(item, 1));
-    slab = std::min(std::min(slab, items), std::max<int64_t>(1, 2147483647ll / a.n_seg));
-    // several slabs in flight are worth it from about two waves of the evaluation's CTAs each and
-    // some milliseconds of sampling (10^9 Philox blocks)
-    const int64_t wave = 2 * sms;
-    if (items >= 4 * wave && slab > (items + 3) / 4 && bytes <= budget && (double)nb * t * ((a.k + 3) / 4) >= 1e9) {
-        slab = (std::max<int64_t>(2 * wave, (items + 3) / 4) + a.n_chunks - 1) / a.n_chunks * a.n_chunks;
-        slab = std::min(slab, items);
-    }
+    const int64_t slab = ef::slab_items_of(nb, a.n_chunks, a.n_seg, item, img, slab_bytes, sms, (double)nb * t * ((a.k + 3) / 4));
     a.slab_items = slab;
-    const bool two = items > slab;
+    const bool two = std::max<int64_t>(nb, 1) * a.n_chunks > slab;
     const size_t samples = item ? (ef::approx_sample_bytes(a, slab, &o_ent, &o_sum, &o_cnt) + 255) / 256 * 256 : 0;
-    const size_t images = ((size_t)std::min<int64_t>(std::max<int64_t>(nb, 1), slab / a.n_chunks + 2) * img + 255) / 256 * 256;
+    const size_t images = ((size_t)ef::slab_images(nb, slab, a.n_chunks) * img + 255) / 256 * 256;
     EF_CK(c->daSamples.ensure((two ? 2 : 1) * samples));
     EF_CK(c->daImage.ensure((two ? 2 : 1) * images));
     if (two) {

@@ -1,4 +1,5 @@
-"""Order of a call's slabs on two streams (csrc/ef_slabs.h), compiled with the host compiler."""
+"""Size and order of a call's slabs on two streams (csrc/ef_slabs.h), compiled with the host compiler."""
+import itertools
 import os
 import shutil
 import subprocess
@@ -12,6 +13,13 @@ MAIN = r"""
 #include <cstdlib>
 #include "ef_slabs.h"
 int main(int argc, char** argv) {
+    if (argc > 6) {  // nb, n_chunks, n_seg, item, image, budget, sms, blocks
+        const int64_t nb = atoll(argv[1]), nc = atoll(argv[2]);
+        const int64_t slab = ef::slab_items_of(nb, nc, atoll(argv[3]), atoll(argv[4]), atoll(argv[5]), atoll(argv[6]), atoll(argv[7]),
+                                               atof(argv[8]));
+        printf("%ld %ld\n", (long)slab, (long)ef::slab_images(nb, slab, nc));
+        return 0;
+    }
     const long items = atol(argv[1]), slab = atol(argv[2]), two = atol(argv[3]), bad = atol(argv[4]);
     long n = 0;
     const auto step = [&](const char* what) {
@@ -52,3 +60,17 @@ def test_a_failed_launch_still_joins(run):
     assert run(9, 3, 1, 5) == ["fork", "0+3@0", "3+3@1", "6+3@0", "join", "105"]
     assert run(9, 3, 1, 1) == ["fork", "101"]  # nothing is on the side stream yet
     assert run(9, 3, 0, 2) == ["0+3@0", "3+3@0", "102"]
+
+
+def test_slabs_stay_within_the_budget(run):
+    budget, sms = 512 << 20, 152
+    seen = set()
+    for nb, nc, item, image in itertools.product((1, 7, 300, 1776, 1900, 8192), (1, 3, 12, 1824), (0, 9000, 290_000, 900_000),
+                                                 (400, 50_000, 200_000)):
+        for blocks in (1e6, 1e10):
+            slab, images = map(int, run(nb, nc, 4, item, image, budget, sms, blocks))
+            assert 1 <= slab <= nb * nc and slab * item + images * image <= budget
+            whole = image + item * nc <= budget - 2 * image
+            assert not whole or slab % nc == 0  # whole bitstrings where one fits
+            seen.add((whole, slab < nb * nc, blocks >= 1e9 and slab >= 4 * sms))
+    assert {s[0] for s in seen} == {True, False} and any(s[1] for s in seen)
