@@ -19,6 +19,7 @@
 #include <cmath>
 #include <complex>
 #include <map>
+#include <mutex>
 #include <cstring>
 #include <new>
 #include <string>
@@ -64,26 +65,140 @@ struct CP {
     bool phase_only;   // changes no probability (see the gate classes in prepare)
 };
 
+// ------------------------------------------------------------------ workspace of a call
+// The samples and images of a Raw Estimate call (up to 512 MiB a slab, two slabs) are
+// needed while it runs only. They come, in the order of the call's stream, from one
+// pool per device, so that memory goes with the calls in flight and not with the
+// circuits that exist: 16 circuits that had made one call each held 16 GiB. The pool
+// keeps at most kPoolKeep between calls and, once no circuit is left, kPoolIdle. Work
+// captured into a graph owns its allocation. Up to kOwnWork a circuit keeps them
+// beside its partial sums (taking and giving back cost a host call of 117 us another
+// 7), in a buffer that comes from the pool too: 3.5 MB by cudaMalloc cost a new
+// circuit's first call 60 us of 430.
+constexpr size_t kOwnWork = (size_t)8 << 20;
+constexpr uint64_t kPoolKeep = (uint64_t)2 << 30;
+constexpr uint64_t kPoolIdle = (uint64_t)64 << 20;
+constexpr int kMaxDevices = 64;
+std::mutex g_pool_mu;
+cudaMemPool_t g_pool[kMaxDevices] = {};
+int g_pool_circuits = 0;
+
+// Memory that no call holds goes back to the device, all but `keep` bytes of it.
+void pool_trim(uint64_t keep) {
+    for (cudaMemPool_t p : g_pool)
+        if (p) cudaMemPoolTrimTo(p, keep);
+}
+
+cudaError_t pool_of_device(cudaMemPool_t* out) {
+    int dev = -1;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+    std::lock_guard<std::mutex> lock(g_pool_mu);
+    if (!g_pool[dev]) {
+        cudaMemPoolProps props{};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = dev;
+        cudaMemPool_t p = nullptr;
+        if ((e = cudaMemPoolCreate(&p, &props)) != cudaSuccess) return e;
+        uint64_t keep = kPoolKeep;
+        int off = 0;  // memory freed on another stream is not worth waiting for
+        e = cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep);
+        if (e == cudaSuccess) e = cudaMemPoolSetAttribute(p, cudaMemPoolReuseAllowInternalDependencies, &off);
+        if (e != cudaSuccess) {
+            cudaMemPoolDestroy(p);
+            return e;
+        }
+        g_pool[dev] = p;
+    }
+    *out = g_pool[dev];
+    return cudaSuccess;
+}
+
+// Memory of the pool from take() to the end of the scope, in the order of stream s.
+struct CallMemory {
+    unsigned char* p = nullptr;
+    cudaStream_t s = nullptr;
+    cudaError_t take(size_t bytes, cudaStream_t stream) {
+        cudaMemPool_t pool = nullptr;
+        cudaError_t e = pool_of_device(&pool);
+        if (e != cudaSuccess) return e;
+        s = stream;
+        void* q = nullptr;
+        e = cudaMallocFromPoolAsync(&q, std::max<size_t>(bytes, 256), pool, s);
+        if (e == cudaSuccess) p = static_cast<unsigned char*>(q);
+        return e;
+    }
+    ~CallMemory() {
+        if (p) cudaFreeAsync(p, s);
+    }
+};
+
+// cudaMalloc, once more without what the pool keeps if there is no room.
+cudaError_t device_malloc(void** p, size_t bytes) {
+    cudaError_t e = cudaMalloc(p, bytes);
+    if (e != cudaErrorMemoryAllocation) return e;
+    cudaGetLastError();
+    {
+        std::lock_guard<std::mutex> lock(g_pool_mu);
+        pool_trim(0);
+    }
+    return cudaMalloc(p, bytes);
+}
+
 // A device buffer that only grows. Every reallocation bumps the owner's
 // workspace epoch, so that captured work holding the old address can tell.
 struct DBuf {
     void* p = nullptr;
     size_t bytes = 0;
     uint64_t* epoch = nullptr;
+    bool pooled = false;
+    std::vector<void*> left;  // pool memory that could not be given back under capture
     cudaError_t ensure(size_t want) {
         if (want <= bytes) return cudaSuccess;
-        if (p) cudaFree(p);
+        if (p && pooled) left.push_back(p);
+        else if (p) cudaFree(p);
         p = nullptr;
         bytes = 0;
+        pooled = false;
         if (epoch) ++*epoch;
-        cudaError_t e = cudaMalloc(&p, std::max<size_t>(want, 256));
+        cudaError_t e = device_malloc(&p, std::max<size_t>(want, 256));
         if (e == cudaSuccess) bytes = std::max<size_t>(want, 256);
         return e;
     }
+    // The same from the pool of the device, in the order of stream s, on which the owner's
+    // earlier work has run and its next work runs. (Under capture the memory would belong to
+    // the graph: by cudaMalloc.)
+    cudaError_t ensure_pooled(size_t want, cudaStream_t s) {
+        if (want <= bytes) return cudaSuccess;
+        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+        cudaError_t e = cudaStreamIsCapturing(s, &capture);
+        if (e != cudaSuccess) return e;
+        if (capture != cudaStreamCaptureStatusNone) return ensure(want);
+        CallMemory before, m;
+        before.s = s;
+        before.p = pooled ? static_cast<unsigned char*>(p) : nullptr;  // given back after the work on s
+        if (p && !pooled) cudaFree(p);
+        p = nullptr;
+        bytes = 0;
+        if (epoch) ++*epoch;
+        e = m.take(want, s);
+        if (e != cudaSuccess) return e;
+        p = m.p;
+        bytes = std::max<size_t>(want, 256);
+        pooled = true;
+        m.p = nullptr;
+        return cudaSuccess;
+    }
     void release() {
+        if (pooled || !left.empty()) cudaDeviceSynchronize();  // cudaFree does not wait for pool memory
+        for (void* q : left) cudaFree(q);
+        left.clear();
         if (p) cudaFree(p);
         p = nullptr;
         bytes = 0;
+        pooled = false;
     }
     template <typename T> T* as() const { return reinterpret_cast<T*>(p); }
 };
@@ -188,7 +303,7 @@ struct ef_circuit {
 
     bool dirty = true;
     DBuf dWS, dWS32, dWSFF, dList, dListCount, dRecomp, dDedup, dBits, dOut, dErr, dGradP, dGrad, dPbar, dSums;
-    DBuf daT, daq, daq32, dalayer, damodes, dagpair, daPart, dCounters, daList, daSamples, daImage;
+    DBuf daT, daq, daq32, dalayer, damodes, dagpair, daCall, dCounters;
     cudaStream_t own_stream = nullptr;
     ef::SideStream side;  // a second slab of a Raw Estimate call
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
@@ -208,11 +323,13 @@ struct ef_circuit {
     template <typename F> void for_each_buf(F f) {
         for (int b = 0; b < ef::kMaxBlocks; ++b) blk[b].for_each_buf(f);
         for (DBuf* d : {&dWS, &dWS32, &dWSFF, &dList, &dListCount, &dRecomp, &dDedup, &dBits, &dOut, &dErr, &dGradP, &dGrad, &dPbar, &dSums, &daT,
-                        &daq, &daq32, &dalayer, &damodes, &dagpair, &daPart, &dCounters, &daList, &daSamples, &daImage})
+                        &daq, &daq32, &dalayer, &damodes, &dagpair, &daCall, &dCounters})
             f(*d);
     }
     ef_circuit() {
         for_each_buf([this](DBuf& d) { d.epoch = &ws_epoch; });
+        std::lock_guard<std::mutex> lock(g_pool_mu);
+        ++g_pool_circuits;
     }
     ~ef_circuit() {
         for_each_buf([](DBuf& d) { d.release(); });
@@ -222,6 +339,8 @@ struct ef_circuit {
         if (side.fork) cudaEventDestroy(side.fork);
         if (side.join) cudaEventDestroy(side.join);
         if (side.stream) cudaStreamDestroy(side.stream);
+        std::lock_guard<std::mutex> lock(g_pool_mu);
+        if (--g_pool_circuits == 0) pool_trim(kPoolIdle);
     }
 };
 
@@ -1554,7 +1673,27 @@ ef::ApproxDev approx_dev_for(const ef_circuit* c, const ef::ApproxDev& base, boo
     return a;
 }
 
-int approx_setup(ef_circuit* c, int64_t nb, int64_t t, uint64_t seed, uint64_t base, ef::ApproxDev& a) {
+// Layout of a call's samples (K form) and images: one set of both or, with several
+// slabs, two, the samples first.
+struct ApproxWork {
+    size_t samples = 0, images = 0;               // bytes of a set
+    size_t entries = 0, sums = 0, counts = 0;     // offsets in the samples
+    int sets = 1;
+    bool own = false;                             // bound already: part of the circuit's buffer
+    size_t bytes() const { return sets * (samples + images); }
+};
+
+void approx_bind(ef::ApproxDev& a, const ApproxWork& w, unsigned char* p) {
+    if (w.samples) {
+        a.codes = reinterpret_cast<uint16_t*>(p);
+        a.entries = reinterpret_cast<uint4*>(p + w.entries);
+        a.hsums = reinterpret_cast<float*>(p + w.sums);
+        a.seg_multi = reinterpret_cast<int*>(p + w.counts);
+    }
+    a.img = p + w.sets * w.samples;
+}
+
+int approx_setup(ef_circuit* c, int64_t nb, int64_t t, uint64_t seed, uint64_t base, cudaStream_t s, ef::ApproxDev& a, ApproxWork& work) {
     if (!c->approx_ok) return fail(EF_EUNSUPPORTED, c->approx_why);
     const bool fp64 = c->opt.precision == EF_PREC_FP64;
     if (fp64)
@@ -1667,11 +1806,6 @@ int approx_setup(ef_circuit* c, int64_t nb, int64_t t, uint64_t seed, uint64_t b
     }
     a.tol = c->opt.tol;
     a.p_floor = c->p_floor;
-    EF_CK(c->daPart.ensure((size_t)std::max<int64_t>(nb, 1) * a.n_chunks * ef::kApproxPartStride * sizeof(double)));
-    EF_CK(c->dCounters.ensure(8 * sizeof(unsigned long long)));
-    EF_CK(c->daList.ensure(((size_t)std::max<int64_t>(nb, 1) + 4) * sizeof(int)));
-    a.part = c->daPart.as<double>();
-    a.counters = c->dCounters.as<unsigned long long>();
     for (int b = 0; b < c->nblocks; ++b) {
         HostBlock& B = c->blk[b];
         a.blk[b].n = B.n;
@@ -1694,36 +1828,48 @@ int approx_setup(ef_circuit* c, int64_t nb, int64_t t, uint64_t seed, uint64_t b
     const ef::ApproxDev first = approx_dev_for(c, a, fp64);
     const ef::ApproxDev redo = c->opt.precision == EF_PREC_AUTO ? approx_dev_for(c, a, true) : first;
     const int64_t img = std::max(first.img_bytes, redo.img_bytes);
-    size_t o_ent, o_sum, o_cnt;
-    const int64_t item = first.kform || redo.kform ? (int64_t)ef::approx_sample_bytes(a, 1, &o_ent, &o_sum, &o_cnt) : 0;
+    work = ApproxWork{};
+    const auto sample_bytes = [&](int64_t n) { return (int64_t)ef::approx_sample_bytes(a, n, &work.entries, &work.sums, &work.counts); };
+    const int64_t item = first.kform || redo.kform ? sample_bytes(1) : 0;
     const int64_t slab = ef::slab_items_of(nb, a.n_chunks, a.n_seg, item, img, slab_bytes, sms, (double)nb * t * ((a.k + 3) / 4));
     a.slab_items = slab;
     const bool two = std::max<int64_t>(nb, 1) * a.n_chunks > slab;
-    const size_t samples = item ? (ef::approx_sample_bytes(a, slab, &o_ent, &o_sum, &o_cnt) + 255) / 256 * 256 : 0;
-    const size_t images = ((size_t)ef::slab_images(nb, slab, a.n_chunks) * img + 255) / 256 * 256;
-    EF_CK(c->daSamples.ensure((two ? 2 : 1) * samples));
-    EF_CK(c->daImage.ensure((two ? 2 : 1) * images));
+    work.samples = item ? ((size_t)sample_bytes(slab) + 255) / 256 * 256 : 0;
+    work.images = ((size_t)ef::slab_images(nb, slab, a.n_chunks) * img + 255) / 256 * 256;
     if (two) {
         if (!c->side.stream) {
             EF_CK(cudaStreamCreateWithFlags(&c->side.stream, cudaStreamNonBlocking));
             EF_CK(cudaEventCreateWithFlags(&c->side.fork, cudaEventDisableTiming));
             EF_CK(cudaEventCreateWithFlags(&c->side.join, cudaEventDisableTiming));
         }
-        a.alt_samples = (int64_t)samples;
-        a.alt_img = (int64_t)images;
+        work.sets = 2;
+        a.alt_samples = (int64_t)work.samples;
+        a.alt_img = (int64_t)work.images;
         int least = 0, greatest = 0;
         EF_CK(cudaDeviceGetStreamPriorityRange(&least, &greatest));
         a.eval_priority = greatest;
     }
-    unsigned char* sp = c->daSamples.as<unsigned char>();
-    if (item) {
-        a.codes = reinterpret_cast<uint16_t*>(sp);
-        a.entries = reinterpret_cast<uint4*>(sp + o_ent);
-        a.hsums = reinterpret_cast<float*>(sp + o_sum);
-        a.seg_multi = reinterpret_cast<int*>(sp + o_cnt);
-    }
-    a.img = c->daImage.as<unsigned char>();
+    // one buffer of the circuit: partial sums, the flagged list and, if small, samples and images
+    const auto up256 = [](size_t x) { return (x + 255) / 256 * 256; };
+    const size_t bits = (size_t)std::max<int64_t>(nb, 1);
+    const size_t part = up256(bits * a.n_chunks * ef::kApproxPartStride * sizeof(double)), list = up256((bits + 4) * sizeof(int));
+    work.own = work.bytes() <= kOwnWork;
+    EF_CK(c->daCall.ensure_pooled(part + list + (work.own ? work.bytes() : 0), s));
+    EF_CK(c->dCounters.ensure(8 * sizeof(unsigned long long)));
+    unsigned char* p = c->daCall.as<unsigned char>();
+    a.part = reinterpret_cast<double*>(p);
+    a.flagged = reinterpret_cast<int*>(p + part);
+    a.counters = c->dCounters.as<unsigned long long>();
+    if (work.own) approx_bind(a, work, p + part + list);
     a = approx_dev_for(c, a, fp64);
+    return EF_OK;
+}
+
+// Samples and images of a single call, until `mem` ends.
+int approx_memory(ef::ApproxDev& a, const ApproxWork& work, CallMemory& mem, cudaStream_t s) {
+    if (work.own) return EF_OK;
+    EF_CK(mem.take(work.bytes(), s));
+    approx_bind(a, work, mem.p);
     return EF_OK;
 }
 
@@ -1734,7 +1880,7 @@ int approx_enqueue(ef_circuit* c, const ef::ApproxDev& a, const uint64_t* d_bits
                    double* d_err, cudaStream_t s, ef::LaunchStats& st) {
     const bool fp64 = c->opt.precision == EF_PREC_FP64;
     const bool autofix = c->opt.precision == EF_PREC_AUTO && ef::approx_eta_template(a) <= ef::kMaxApproxEta64;
-    int* list = c->daList.as<int>();
+    int* list = a.flagged;
     int* list_count = list + std::max<int64_t>(a.nb, 1);
     EF_CK(cudaMemsetAsync(a.counters, 0, 8 * sizeof(unsigned long long), s));
     EF_CK(cudaMemsetAsync(list_count, 0, sizeof(int), s));
@@ -1762,7 +1908,11 @@ int approx_dev(ef_circuit* c, const uint64_t* d_bits, int64_t nb, int64_t t, uin
     c->stats.logical_branch_dets = nb * t;
     if (nb == 0) return EF_OK;
     ef::ApproxDev a;
-    rc = approx_setup(c, nb, t, seed, base, a);
+    ApproxWork work;
+    rc = approx_setup(c, nb, t, seed, base, s, a, work);
+    if (rc) return rc;
+    CallMemory mem;
+    rc = approx_memory(a, work, mem, s);
     if (rc) return rc;
     ef::LaunchStats st;
     rc = approx_enqueue(c, a, d_bits, d_out, d_se, d_err, s, st);
@@ -1866,7 +2016,11 @@ int estimate_host(ef_circuit* c, const uint64_t* bits, int64_t nb, double eps, d
             int rc = begin_call(c, s, 2);
             if (rc) return rc;
             ef::ApproxDev a;
-            rc = approx_setup(c, ng, t, seed_r, 0, a);
+            ApproxWork work;
+            rc = approx_setup(c, ng, t, seed_r, 0, s, a, work);
+            if (rc) return rc;
+            CallMemory mem;
+            rc = approx_memory(a, work, mem, s);
             if (rc) return rc;
             a.gidx = didx.as<uint64_t>();
             ef::LaunchStats st;
@@ -2215,12 +2369,10 @@ int ef_circuit_get_stats(ef_circuit* c, ef_stats* st) {
 // declares at file scope. It is for callers that must not have a library
 // allocate device memory during their run (see extraferm.h).
 
-#include <mutex>
-
 namespace {
 
 constexpr size_t kNoAllocBytes = (size_t)64 << 20;  // 64 MiB per GPU, held until the process exits
-constexpr int kNoAllocMaxDevices = 64;
+constexpr int kNoAllocMaxDevices = kMaxDevices;
 
 // File-scope scratch. In host code this name is only a stand-in for the
 // device symbol; kernels get its device address from cudaGetSymbolAddress.
@@ -2445,6 +2597,8 @@ struct ef_batch {
         int mode = 0;  // 1 exact via the work queues, 2 exact on its own launches, 3 Raw Estimate
         ExactBuffers eb{};
         ef::ApproxDev a{};
+        ApproxWork work;  // Raw Estimate: in work[side] of the batch
+        int side = 0;
         const uint64_t* bits = nullptr;
         int64_t nb = 0;
         double* out = nullptr;
@@ -2460,6 +2614,7 @@ struct ef_batch {
     std::vector<ef::QueueEntry> entries;
     std::vector<std::pair<int, int>> entry_src;  // (item, block) of each entry
     DBuf dEntries, dHeads;
+    std::vector<DBuf> work;    // per side stream: samples and images of the Raw Estimate circuits that take turns on it
     std::map<int, int> tuned;  // eta -> pattern-chunk log2
     int64_t launches = 0;
     int64_t logical = 0;
@@ -2472,6 +2627,7 @@ struct ef_batch {
         if (cap) cudaStreamDestroy(cap);
         dEntries.release();
         dHeads.release();
+        for (DBuf& w : work) w.release();
     }
 };
 
@@ -2526,8 +2682,9 @@ int batch_enqueue(ef_batch* bt, cudaStream_t s, ef::LaunchStats& st) {
     for (size_t i = 0; i < bt->items.size(); ++i) {
         ef_batch::Item& it = bt->items[i];
         if (it.mode != 3 || it.nb == 0) continue;
-        int rc = approx_enqueue(bt->cs[i], it.a, it.bits, it.out, nullptr, nullptr, bt->side[rr++ % ns], st);
+        int rc = approx_enqueue(bt->cs[i], it.a, it.bits, it.out, nullptr, nullptr, bt->side[it.side], st);
         if (rc) return rc;
+        ++rr;
     }
     for (size_t i = 0; i < bt->items.size(); ++i) {
         ef_batch::Item& it = bt->items[i];
@@ -2711,13 +2868,27 @@ extern "C" int ef_batch_prob_dev(ef_batch* bt, const uint64_t* const* d_bits, co
         } else {
             rc = begin_call(c, s, 2);
             if (rc) return rc;
-            rc = approx_setup(c, nb[i], n_traj[i], seed, 0, it.a);
+            rc = approx_setup(c, nb[i], n_traj[i], seed, 0, s, it.a, it.work);
             if (rc) return rc;
             it.mode = 3;
             bt->logical += nb[i] * n_traj[i];
         }
     }
     EF_CK(cudaStreamSynchronize(s));
+    // Raw Estimate circuits take the side streams in turn, and the workspace of theirs
+    bt->work.resize(bt->side.size());
+    int turn = 0;
+    for (int pass = 0; pass < 2; ++pass)
+        for (ef_batch::Item& it : bt->items) {
+            if (it.mode != 3 || it.nb == 0) continue;
+            if (pass == 0) it.side = turn++ % (int)bt->side.size();
+            if (it.work.own) continue;
+            if (pass == 0) {
+                EF_CK(bt->work[it.side].ensure(it.work.bytes()));
+            } else {
+                approx_bind(it.a, it.work, bt->work[it.side].as<unsigned char>());
+            }
+        }
     // work-queue classes by particle count
     bt->classes.clear();
     bt->entries.clear();

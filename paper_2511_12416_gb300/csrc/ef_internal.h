@@ -163,6 +163,7 @@ struct ApproxDev {
     uint64_t inactive0, inactive1;
     int64_t t;
     int64_t nb;              // bitstrings of the call
+    int* flagged;            // room for the bitstrings that the FP32 pass flags and, behind it, for their number
     const int* list;         // null: every bitstring; else the listed bitstrings (FP64 redo)
     const int* list_count;   //   their number (device)
     int traj_per_cta;
