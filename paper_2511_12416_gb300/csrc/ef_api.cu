@@ -1007,11 +1007,18 @@ struct ExactBuffers {
     int mark_words;
 };
 
-// Equal bitstrings are looked for from this many bitstrings on. The search runs
-// beside the branch builder and costs a clearing of its table (about 2 us); 1500
-// uniform bitstrings of the 32-qubit workload, 6 % of them repeats on a block, just
-// pay for it.
-constexpr int64_t kDedupMin = 1024;
+// Equal bitstrings of two mode blocks are looked for in sets of at least 1024
+// bitstrings and 2^17 minors. The search costs about 7 us a call (clearing, its
+// chain of dependent loads beside the builder, a column looked up by the combines)
+// and 0.1 ns a bitstring; FP32 minors cost 0.015 (2 and 4 particles) to 0.065 ns
+// (8). Uniform sets over 16 modes and 8 particles a spin, searched / not, us: 4
+// patterns a block, 2000 bitstrings 47 / 36 (left out by the rule), 20,000 79 / 77,
+// 10^5 209 / 246, 10^6 1581 / 2124; 64 patterns, 2000 72 / 63, 20,000 201 / 280; 256
+// patterns, 2000 146 / 146, 20,000 565 / 894. Sets with more repeats gain sooner.
+bool search_for_equal(const ef_circuit* c, int64_t nb) {
+    if (c->nblocks != 2 || nb < 1024) return false;
+    return (double)nb * (std::ldexp(1.0, c->blk[0].r) + std::ldexp(1.0, c->blk[1].r)) >= 131072.0;
+}
 
 // EF_PREC_AUTO redoes single determinants (rather than whole bitstrings) when
 // the thread-per-minor FP64 kernel covers every block and the combine can hold
@@ -1182,7 +1189,7 @@ int exact_enqueue_build(ef_circuit* c, const ExactBuffers& eb, const uint64_t* b
     ef::DedupDev d = eb.dedup;
     d.bits = bits;
     d.nb = nbb;
-    if (d.table[0]) EF_CK(cudaMemsetAsync(d.table[0], 0, eb.dedup_clear, s));
+    if (d.table[0]) EF_CK(ef::launch_dedup_clear(d.table[0], eb.dedup_clear, s, st));
     const bool counters = c->opt.precision == EF_PREC_AUTO || d.table[0];  // nothing else reads them
     EF_CK(ef::launch_build_branches(eb.blk[0], eb.blk[1], c->nblocks, !fp64_only, counters ? eb.count : nullptr, eb.recomp,
                                     d.table[0] ? &d : nullptr, s, st));
@@ -1282,7 +1289,7 @@ int run_exact(ef_circuit* c, const ExactBuffers& eb, const uint64_t* d_bits, int
             ef::DedupDev d = eb.dedup;
             d.bits = bits;
             d.nb = nbb;
-            EF_CK(cudaMemsetAsync(d.table[0], 0, eb.dedup_clear, s));
+            EF_CK(ef::launch_dedup_clear(d.table[0], eb.dedup_clear, s, st));
             EF_CK(ef::launch_dedup(eb.blk[0], eb.blk[1], d, s, st));
         }
         if (c->timed && off == 0) EF_CK(cudaEventRecord(c->ev0, s));
@@ -1389,7 +1396,7 @@ int exact_dev(ef_circuit* c, const uint64_t* d_bits, int64_t nb, double* d_out, 
     c->stats.logical_branch_dets = nb * (int64_t)std::ldexp(1.0, (int)c->cps.size());
     if (nb == 0) return EF_OK;
     ExactBuffers eb;
-    rc = exact_buffers(c, exact_batch(c, nb, (size_t)2 << 30), c->nblocks == 2 && nb >= kDedupMin, eb);
+    rc = exact_buffers(c, exact_batch(c, nb, (size_t)2 << 30), search_for_equal(c, nb), eb);
     if (rc) return rc;
     ef::LaunchStats st;
     return run_exact(c, eb, d_bits, nb, d_out, d_err, s, st);

@@ -170,51 +170,91 @@ __device__ __forceinline__ float4 cf_of_d(double2 a) {
 // workload 54 % are distinct on 8 of 16 modes; sets sampled from a state or built as
 // products of alpha and beta strings repeat far more. Which of the equal ones
 // stands for them depends on the order of arrival, the results do not.
+// A warp takes 32 bitstrings of a block a turn (turns first, first + step, ...); those
+// that are the first of their kind get their places by one addition a warp, and a
+// place of the table is read before it is exchanged: sets of few distinct
+// bitstrings would else queue at as few addresses.
 __device__ __forceinline__ void dedup_range(const ExactBlockDev& B0, const ExactBlockDev& B1, const DedupDev& D, int64_t first,
                                             int64_t step) {
-    for (int64_t x = first; x < 2 * D.nb; x += step) {
-        const int blk = x >= D.nb ? 1 : 0;
-        const int64_t b = x - (blk ? D.nb : 0);
+    const int lane = threadIdx.x & 31;
+    const int64_t turns = (D.nb + 31) >> 5;  // of a block
+    for (int64_t x = first; x < 2 * turns; x += step) {
+        const int blk = x >= turns ? 1 : 0;
+        const int64_t b = ((x - (blk ? turns : 0)) << 5) + lane;
         const uint64_t m0 = blk ? B1.mask0 : B0.mask0, m1 = blk ? B1.mask1 : B0.mask1;
-        const uint64_t w0 = D.bits[2 * b] & m0, w1 = D.bits[2 * b + 1] & m1;
-        // a multiplicative mix of both words; the table is at most half full
-        uint64_t h = (w0 * 0x9E3779B97F4A7C15ull) ^ (w1 * 0xC2B2AE3D27D4EB4Full);
-        h ^= h >> 32;
-        h *= 0x9E3779B97F4A7C15ull;
-        uint32_t at = (uint32_t)(h >> 32) & D.hmask;
-        int* tab = blk ? D.table[1] : D.table[0];
         int* ucol = blk ? D.ucol[1] : D.ucol[0];
         uint64_t* ubits = blk ? D.ubits[1] : D.ubits[0];
-        int r = (int)b;
-        for (uint32_t probe = 0; probe <= D.hmask; ++probe) {
-            const int old = atomicCAS(&tab[at], 0, (int)b + 1);
-            if (old == 0) {  // the first of its kind
-                const int u = atomicAdd(&D.ucount[blk], 1);
-                ucol[b] = u;
-                ubits[2 * u] = w0;
-                ubits[2 * u + 1] = w1;
-                break;
+        uint64_t w0 = 0, w1 = 0;
+        bool fresh = false;
+        if (b < D.nb) {
+            w0 = D.bits[2 * b] & m0;
+            w1 = D.bits[2 * b + 1] & m1;
+            // a multiplicative mix of both words; the table is at most half full
+            uint64_t h = (w0 * 0x9E3779B97F4A7C15ull) ^ (w1 * 0xC2B2AE3D27D4EB4Full);
+            h ^= h >> 32;
+            h *= 0x9E3779B97F4A7C15ull;
+            uint32_t at = (uint32_t)(h >> 32) & D.hmask;
+            int* tab = blk ? D.table[1] : D.table[0];
+            int r = (int)b;
+            for (uint32_t probe = 0; probe <= D.hmask; ++probe) {
+                int old = __ldcg(&tab[at]);
+                if (old == 0) old = atomicCAS(&tab[at], 0, (int)b + 1);
+                if (old == 0) {  // the first of its kind
+                    fresh = true;
+                    break;
+                }
+                if ((D.bits[2 * (int64_t)(old - 1)] & m0) == w0 && (D.bits[2 * (int64_t)(old - 1) + 1] & m1) == w1) {
+                    r = old - 1;
+                    break;
+                }
+                at = (at + 1) & D.hmask;
             }
-            if ((D.bits[2 * (old - 1)] & m0) == w0 && (D.bits[2 * (old - 1) + 1] & m1) == w1) {
-                r = old - 1;
-                break;
-            }
-            at = (at + 1) & D.hmask;
+            (blk ? D.rep[1] : D.rep[0])[b] = r;
         }
-        (blk ? D.rep[1] : D.rep[0])[b] = r;
+        const unsigned who = __ballot_sync(0xffffffffu, fresh);
+        if (!who) continue;
+        int u = 0;
+        if (lane == 0) u = atomicAdd(&D.ucount[blk], __popc(who));
+        u = __shfl_sync(0xffffffffu, u, 0) + __popc(who & ((1u << lane) - 1u));
+        if (fresh) {
+            ucol[b] = u;
+            ubits[2 * (int64_t)u] = w0;
+            ubits[2 * (int64_t)u + 1] = w1;
+        }
     }
+}
+__device__ __forceinline__ void dedup_grid(const ExactBlockDev& B0, const ExactBlockDev& B1, const DedupDev& D) {
+    const int warps = blockDim.x >> 5;
+    dedup_range(B0, B1, D, (int64_t)blockIdx.x * warps + (threadIdx.x >> 5), (int64_t)gridDim.x * warps);
+}
+// The table's clearing, a kernel in the chain of programmatic launches: 2 us less than a memset.
+__global__ void __launch_bounds__(256) k_dedup_clear(uint4* p, int64_t n) {
+    cudaGridDependencySynchronize();  // see launch_pdl
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        p[i] = make_uint4(0u, 0u, 0u, 0u);
+}
+
+cudaError_t launch_dedup_clear(void* p, size_t bytes, cudaStream_t s, LaunchStats& st) {
+    const int64_t n = (int64_t)(bytes / sizeof(uint4));
+    const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, (int64_t)sm_count() * 8));
+    st.launches += 1;
+    return launch_pdl(k_dedup_clear, dim3((unsigned)blocks), dim3(256), 0, s, reinterpret_cast<uint4*>(p), n);
+}
+
+// CTAs of nt threads for the search of nb bitstrings over two blocks
+static unsigned dedup_blocks(int64_t nb, unsigned nt) {
+    return (unsigned)std::max<int64_t>(1, std::min<int64_t>((2 * nb + nt - 1) / nt, (int64_t)sm_count() * 8));
 }
 
 __global__ void __launch_bounds__(256) k_dedup(ExactBlockDev B0, ExactBlockDev B1, DedupDev D) {
     cudaGridDependencySynchronize();  // see launch_pdl
-    dedup_range(B0, B1, D, (int64_t)blockIdx.x * blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x);
+    dedup_grid(B0, B1, D);
 }
 
 cudaError_t launch_dedup(const ExactBlockDev& b0, const ExactBlockDev& b1, const DedupDev& d, cudaStream_t s,
                          LaunchStats& st) {
-    const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>((2 * d.nb + 255) / 256, (int64_t)sm_count() * 8));
     st.launches += 1;
-    return launch_pdl(k_dedup, dim3((unsigned)blocks), dim3(256), 0, s, b0, b1, d);
+    return launch_pdl(k_dedup, dim3(dedup_blocks(d.nb, 256)), dim3(256), 0, s, b0, b1, d);
 }
 
 struct NoDedup {};
@@ -229,7 +269,7 @@ __global__ void __launch_bounds__(512) k_build_branches(ExactBlockDev B0, ExactB
     }
     if constexpr (std::is_same<D, DedupDev>::value)
         if (blockIdx.y == 2) {  // beside the builder, which is mostly latency
-            dedup_range(B0, B1, dedup, (int64_t)blockIdx.x * blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x);
+            dedup_grid(B0, B1, dedup);
             return;
         }
     const ExactBlockDev& B = blockIdx.y ? B1 : B0;
@@ -343,7 +383,9 @@ cudaError_t launch_build_branches(const ExactBlockDev& b0, const ExactBlockDev& 
     if (dedup) {
         if (nblk != 2) return cudaErrorInvalidValue;
         if ((e = raise_dynamic_smem((const void*)k_build_branches<DedupDev>, smem)) != cudaSuccess) return e;
-        return launch_pdl(k_build_branches<DedupDev>, dim3(gx, 3u), dim3(nt), smem, s, b0, bb, want32 ? 1 : 0, count, recomp,
+        // as wide as the builder or the search asks for (the builder's CTAs past 2^r have nothing to do)
+        const unsigned wide = std::max(gx, dedup_blocks(dedup->nb, nt));
+        return launch_pdl(k_build_branches<DedupDev>, dim3(wide, 3u), dim3(nt), smem, s, b0, bb, want32 ? 1 : 0, count, recomp,
                           *dedup);
     }
     if ((e = raise_dynamic_smem((const void*)k_build_branches<NoDedup>, smem)) != cudaSuccess) return e;

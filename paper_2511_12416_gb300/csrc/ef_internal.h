@@ -271,6 +271,8 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
 // bitstrings (dedup; null: does not)
 cudaError_t launch_build_branches(const ExactBlockDev& b0, const ExactBlockDev& b1, int nblk, bool want32, int* count,
                                   unsigned long long* recomp, const DedupDev* dedup, cudaStream_t s, LaunchStats& st);
+// zeroes a search table and what follows it (bytes: a multiple of 16)
+cudaError_t launch_dedup_clear(void* p, size_t bytes, cudaStream_t s, LaunchStats& st);
 cudaError_t launch_dedup(const ExactBlockDev& b0, const ExactBlockDev& b1, const DedupDev& d, cudaStream_t s,
                          LaunchStats& st);
 // FP32 minors of nblk (1 or 2) mode blocks with the same eta in one launch
