@@ -1042,13 +1042,21 @@ size_t det_bytes(const ef_circuit* c) {
            (p != EF_PREC_FP32_MINOR ? sizeof(double2) : 0);
 }
 
-// Bitstrings per batch so that the per-(pattern, bitstring) determinants stay
-// within `budget` bytes.
-int64_t exact_batch(const ef_circuit* c, int64_t nb, size_t budget) {
+// Words of marks per bitstring (see ExactCombineDev).
+int mark_words(const ef_circuit* c) {
+    return per_minor_recompute(c) ? (int)((((int64_t)1 << c->blk[0].r) + ((int64_t)1 << c->blk[1].r) + 31) / 32) : 0;
+}
+
+// Bitstrings per batch so that the per-(pattern, bitstring) determinants, the
+// lists and, with a search for equal bitstrings, its tables (at most four
+// entries a bitstring and block), representatives and marks stay within `budget` bytes.
+int64_t exact_batch(const ef_circuit* c, int64_t nb, size_t budget, bool search) {
     size_t per = 0;
     const size_t each = det_bytes(c) + (per_minor_recompute(c) ? sizeof(int2) : 0);
     for (int b = 0; b < c->nblocks; ++b) per += ((size_t)1 << c->blk[b].r) * each;
     if (per == 0 || nb == 0) return std::max<int64_t>(nb, 1);
+    per += 2 * sizeof(int);
+    if (search) per += (2 * (4 + 2) + (size_t)mark_words(c)) * sizeof(int) + 4 * sizeof(uint64_t);
     return std::max<int64_t>(1, std::min<int64_t>(nb, (int64_t)(budget / per)));
 }
 
@@ -1354,8 +1362,7 @@ int exact_buffers(ef_circuit* c, int64_t cap, bool dedup, ExactBuffers& eb) {
         uint32_t h = 1;
         while ((int64_t)h < 2 * cap) h <<= 1;
         d.hmask = h - 1;
-        if (per_minor_recompute(c))
-            eb.mark_words = (int)((((int64_t)1 << c->blk[0].r) + ((int64_t)1 << c->blk[1].r) + 31) / 32);
+        eb.mark_words = mark_words(c);
         EF_CK(c->dDedup.ensure(((size_t)2 * h + 4 + (4 + (size_t)eb.mark_words) * (size_t)cap) * sizeof(int) +
                                (size_t)cap * 4 * sizeof(uint64_t)));
         d.ubits[0] = c->dDedup.as<uint64_t>();
@@ -1396,7 +1403,8 @@ int exact_dev(ef_circuit* c, const uint64_t* d_bits, int64_t nb, double* d_out, 
     c->stats.logical_branch_dets = nb * (int64_t)std::ldexp(1.0, (int)c->cps.size());
     if (nb == 0) return EF_OK;
     ExactBuffers eb;
-    rc = exact_buffers(c, exact_batch(c, nb, (size_t)2 << 30), search_for_equal(c, nb), eb);
+    const bool search = search_for_equal(c, nb);
+    rc = exact_buffers(c, exact_batch(c, nb, (size_t)2 << 30, search), search, eb);
     if (rc) return rc;
     ef::LaunchStats st;
     return run_exact(c, eb, d_bits, nb, d_out, d_err, s, st);
@@ -2865,7 +2873,7 @@ extern "C" int ef_batch_prob_dev(ef_batch* bt, const uint64_t* const* d_bits, co
             if (!c->exact_ok) return fail(EF_EUNSUPPORTED, "circuit " + std::to_string(i) + ": " + c->exact_why);
             rc = begin_call(c, s, 1);
             if (rc) return rc;
-            const int64_t cap = exact_batch(c, std::max<int64_t>(nb[i], 1), (size_t)2 << 30);
+            const int64_t cap = exact_batch(c, std::max<int64_t>(nb[i], 1), (size_t)2 << 30, false);
             rc = exact_buffers(c, cap, false, it.eb);
             if (rc) return rc;
             bool q = cap >= nb[i] && c->opt.precision != EF_PREC_FP64;

@@ -29,3 +29,23 @@ def test_search_by_the_minors_it_can_spare(lib, onsite, same, nb, searched):
     assert np.array_equal(p[-700:], some)
     distinct = [len(np.unique(x)) for x in (alpha[:40], beta)]
     assert done == (sum(distinct) * minors // 2 if searched else nb * minors)
+
+
+def test_search_tables_count_in_a_slice(lib):
+    """Two patterns a block: a bitstring's tables weigh as much as its determinants, and both
+    stay within the 2 GiB of a slice (14 million bitstrings in one slice took 2.8 GiB)."""
+    torch = pytest.importorskip("torch")
+    c = W.lucj_circuit(16, 8, 8, 1, n_onsite=1, n_same=0, angle_sampler=W.normal_var(0.1), seed=7)
+    base = W.spin_sector_bitstrings(16, 8, 8, 500, np.random.default_rng(3))
+    nb = 14_000_000
+    d = torch.from_numpy(base.view(np.int64)).cuda().repeat(nb // 500, 1).contiguous()
+    out = torch.zeros(nb, dtype=torch.float64, device="cuda")
+    with lib.Circuit(c.n_modes, c.occupation, c.gates) as h:
+        ref = lib.ef_prob_exact(h.handle, base)  # tables and kernels are there
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        lib.ef_prob_exact_dev(h.handle, d.data_ptr(), nb, out.data_ptr(), 0, torch.cuda.current_stream().cuda_stream)
+        torch.cuda.synchronize()
+        used = free - torch.cuda.mem_get_info()[0]
+    assert used <= (2 << 30) + (64 << 20)
+    assert torch.equal(out.view(-1, 500), torch.from_numpy(ref).cuda().expand(nb // 500, 500))
