@@ -52,11 +52,12 @@
  * caller owns every input and output buffer. A circuit owns its device
  * tables and a grow-only device workspace, so the calls on one circuit must
  * be ordered (one host thread at a time, one stream at a time); different
- * circuits are independent. Raw Estimate calls keep 88 bytes per (bitstring, chunk of
- * trajectories) and at most 8 MiB of samples; a call that needs more, 1 GiB at
- * the most, takes it in stream order from a memory pool of the device for as
- * long as it runs. The library keeps at most 2 GiB of the pool between calls
- * and 64 MiB once every circuit is destroyed. A batch holds what the Raw
+ * circuits are independent. Exact calls work through their bitstrings in
+ * slices of at most 2 GiB. Raw Estimate calls keep 88 bytes per (bitstring,
+ * chunk of trajectories) and at most 8 MiB of samples; a call that needs more,
+ * 1 GiB at the most, takes it in stream order from a memory pool of the device
+ * for as long as it runs. The library keeps at most 2 GiB of the pool between
+ * calls and 64 MiB once every circuit is destroyed. A batch holds what the Raw
  * Estimate circuits on each of its four streams need at the most.
  */
 #ifndef EXTRAFERM_H
