@@ -1736,16 +1736,8 @@ int approx_setup(ef_circuit* c, int64_t nb, int64_t t, uint64_t seed, uint64_t b
     a.inactive1 = c->inactive[1];
     a.t = t;
     a.nb = nb;
-    // enough (bitstring, chunk) items for about four waves of three CTAs per SM
     const int64_t sms = ef::sm_count();
     a.sms = (int)sms;
-    const int64_t target = sms * 3 * 4;
-    int64_t chunks = std::max<int64_t>(1, (target + std::max<int64_t>(nb, 1) - 1) / std::max<int64_t>(nb, 1));
-    chunks = std::min<int64_t>(chunks, std::max<int64_t>(1, t / 256));
-    int64_t per = (t + chunks - 1) / chunks;
-    per = (per + 127) / 128 * 128;
-    // (at most 2^25 trajectories per chunk: the samples of one must fit the workspace)
-    a.traj_per_cta = (int)std::min<int64_t>(per, (int64_t)1 << 25);
     {
         // room for the entries of a segment: the expected number of trajectories with two or more
         // flips and eight standard deviations (those past it are sampled again)
@@ -1757,21 +1749,9 @@ int approx_setup(ef_circuit* c, int64_t nb, int64_t t, uint64_t seed, uint64_t b
         const double mean = ef::approx_segment_traj() * std::max(0.0, 1.0 - p0 - p1);
         a.ent_cap = (int)std::min<double>(ef::approx_segment_traj(), std::ceil(mean + 8.0 * std::sqrt(mean)) + 32.0);
     }
-    // A slab (512 MiB, below) of fewer items than two waves of two CTAs per SM is all tail: where
-    // many flips make long items larger than that, they are cut so that a slab holds 12 per SM.
-    // 64 uneven circuits, 10^5 and more trajectories for each of many bitstrings: 42.3 s uncut,
-    // 34.9 s at 6 per SM, 33.7 s at 12, 33.8 s at 24. Cutting the 52-qubit LUCJ circuit's items
-    // too, whose slabs hold 800, costs 4-6 % (6-12 per SM).
-    const int64_t slab_bytes = (int64_t)512 << 20;
-    if (c->kform_ok) {
-        const int64_t seg = (int64_t)4 * ef::approx_segment_traj();
-        const int64_t seg_bytes = seg * (int64_t)sizeof(uint16_t) + 4 * (int64_t)a.ent_cap * (int64_t)sizeof(uint4);
-        if (ef::approx_segments(a.traj_per_cta) * seg_bytes > slab_bytes / (4 * sms)) {
-            const int64_t most = std::max<int64_t>(1, slab_bytes / target / seg_bytes) * seg;
-            const int64_t parts = (t + most - 1) / most;
-            a.traj_per_cta = (int)(((t + parts - 1) / parts + 127) / 128 * 128);
-        }
-    }
+    const int64_t slab_bytes = (int64_t)512 << 20, seg = (int64_t)4 * ef::approx_segment_traj();
+    const int64_t seg_bytes = c->kform_ok ? seg * (int64_t)sizeof(uint16_t) + 4 * (int64_t)a.ent_cap * (int64_t)sizeof(uint4) : 0;
+    a.traj_per_cta = (int)ef::chunk_trajectories(nb, t, sms, seg, seg_bytes, slab_bytes);
     a.n_chunks = (int)((t + a.traj_per_cta - 1) / a.traj_per_cta);
     a.kappa_max = 1e3;
     // K u, the per-trajectory bounds being in units of u = 2^-24. Calibrated

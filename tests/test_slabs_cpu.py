@@ -13,7 +13,12 @@ MAIN = r"""
 #include <cstdlib>
 #include "ef_slabs.h"
 int main(int argc, char** argv) {
-    if (argc > 6) {  // nb, n_chunks, n_seg, item, image, budget, sms, blocks
+    if (argc == 7) {  // nb, t, sms, segment, seg_bytes, slab_bytes
+        printf("%ld\n", (long)ef::chunk_trajectories(atoll(argv[1]), atoll(argv[2]), atoll(argv[3]), atoll(argv[4]), atoll(argv[5]),
+                                                     atoll(argv[6])));
+        return 0;
+    }
+    if (argc > 7) {  // nb, n_chunks, n_seg, item, image, budget, sms, blocks
         const int64_t nb = atoll(argv[1]), nc = atoll(argv[2]);
         const int64_t slab = ef::slab_items_of(nb, nc, atoll(argv[3]), atoll(argv[4]), atoll(argv[5]), atoll(argv[6]), atoll(argv[7]),
                                                atof(argv[8]));
@@ -74,3 +79,14 @@ def test_slabs_stay_within_the_budget(run):
             assert not whole or slab % nc == 0  # whole bitstrings where one fits
             seen.add((whole, slab < nb * nc, blocks >= 1e9 and slab >= 4 * sms))
     assert {s[0] for s in seen} == {True, False} and any(s[1] for s in seen)
+
+
+def test_partial_sums_of_long_calls(run):
+    sms, seg, seg_bytes, slab = 152, 4096, 73_728, 512 << 20  # every trajectory with an entry
+    for nb, t in itertools.product((1, 4, 500, 10_000, 1_000_000), (1, 1000, 68_416, 10 ** 6, 2 ** 32)):
+        cut, uncut = (int(run(nb, t, sms, seg, b, slab)[0]) for b in (seg_bytes, 0))
+        assert cut % 128 == 0 and 128 <= cut <= uncut <= 2 ** 25
+        assert nb * -(-t // cut) <= max(2 ** 24, nb * -(-t // min(uncut, 2 ** 23)))
+        assert -(-cut // seg) * seg_bytes <= slab // 2 + seg_bytes
+        if nb * t <= 2 ** 24 * 3 * seg:  # within that, an item's samples leave room for 12 per SM in a slab
+            assert -(-cut // seg) * seg_bytes <= slab // (4 * sms)
