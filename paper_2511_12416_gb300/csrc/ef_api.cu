@@ -73,36 +73,40 @@ struct CP {
 // keeps at most kPoolKeep between calls and, once no circuit is left, kPoolIdle. Work
 // captured into a graph owns its allocation. Up to kOwnWork a circuit keeps them
 // beside its partial sums (taking and giving back cost a host call of 117 us another
-// 7), in a buffer that comes from the pool too: 3.5 MB by cudaMalloc cost a new
-// circuit's first call 60 us of 430.
+// 7), in a buffer from a second pool where it is small: 3.5 MB by cudaMalloc cost a
+// new circuit's first call 60 us of 430. (A pool reckons what it has lent to what it
+// keeps: with the circuits' buffers in the calls' pool, a call of 13.8 ms beside 400
+// circuits took 15.5 ms, its memory being given back and mapped anew every time.)
 constexpr size_t kOwnWork = (size_t)8 << 20;
 constexpr uint64_t kPoolKeep = (uint64_t)2 << 30;
 constexpr uint64_t kPoolIdle = (uint64_t)64 << 20;
 constexpr int kMaxDevices = 64;
+enum PoolOf { kPoolCalls = 0, kPoolCircuits = 1 };
 std::mutex g_pool_mu;
-cudaMemPool_t g_pool[kMaxDevices] = {};
+cudaMemPool_t g_pool[2][kMaxDevices] = {};
 int g_pool_circuits = 0;
 
-// Memory that no call holds goes back to the device, all but `keep` bytes of it.
+// Memory that no call and no circuit holds goes back to the device, all but `keep` bytes of a pool.
 void pool_trim(uint64_t keep) {
-    for (cudaMemPool_t p : g_pool)
-        if (p) cudaMemPoolTrimTo(p, keep);
+    for (auto& pools : g_pool)
+        for (cudaMemPool_t p : pools)
+            if (p) cudaMemPoolTrimTo(p, keep);
 }
 
-cudaError_t pool_of_device(cudaMemPool_t* out) {
+cudaError_t pool_of_device(PoolOf kind, cudaMemPool_t* out) {
     int dev = -1;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
     std::lock_guard<std::mutex> lock(g_pool_mu);
-    if (!g_pool[dev]) {
+    if (!g_pool[kind][dev]) {
         cudaMemPoolProps props{};
         props.allocType = cudaMemAllocationTypePinned;
         props.location.type = cudaMemLocationTypeDevice;
         props.location.id = dev;
         cudaMemPool_t p = nullptr;
         if ((e = cudaMemPoolCreate(&p, &props)) != cudaSuccess) return e;
-        uint64_t keep = kPoolKeep;
+        uint64_t keep = kind == kPoolCalls ? kPoolKeep : kPoolIdle;
         int off = 0;  // memory freed on another stream is not worth waiting for
         e = cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep);
         if (e == cudaSuccess) e = cudaMemPoolSetAttribute(p, cudaMemPoolReuseAllowInternalDependencies, &off);
@@ -110,19 +114,19 @@ cudaError_t pool_of_device(cudaMemPool_t* out) {
             cudaMemPoolDestroy(p);
             return e;
         }
-        g_pool[dev] = p;
+        g_pool[kind][dev] = p;
     }
-    *out = g_pool[dev];
+    *out = g_pool[kind][dev];
     return cudaSuccess;
 }
 
-// Memory of the pool from take() to the end of the scope, in the order of stream s.
+// Memory of a pool from take() to the end of the scope, in the order of stream s.
 struct CallMemory {
     unsigned char* p = nullptr;
     cudaStream_t s = nullptr;
-    cudaError_t take(size_t bytes, cudaStream_t stream) {
+    cudaError_t take(PoolOf kind, size_t bytes, cudaStream_t stream) {
         cudaMemPool_t pool = nullptr;
-        cudaError_t e = pool_of_device(&pool);
+        cudaError_t e = pool_of_device(kind, &pool);
         if (e != cudaSuccess) return e;
         s = stream;
         void* q = nullptr;
@@ -167,9 +171,9 @@ struct DBuf {
         if (e == cudaSuccess) bytes = std::max<size_t>(want, 256);
         return e;
     }
-    // The same from the pool of the device, in the order of stream s, on which the owner's
+    // The same from the circuits' pool, in the order of stream s, on which the owner's
     // earlier work has run and its next work runs. (Under capture the memory would belong to
-    // the graph: by cudaMalloc.)
+    // the graph: by cudaMalloc, as large buffers.)
     cudaError_t ensure_pooled(size_t want, cudaStream_t s) {
         if (want <= bytes) return cudaSuccess;
         cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
@@ -177,13 +181,19 @@ struct DBuf {
         if (e != cudaSuccess) return e;
         if (capture != cudaStreamCaptureStatusNone) return ensure(want);
         CallMemory before, m;
-        before.s = s;
-        before.p = pooled ? static_cast<unsigned char*>(p) : nullptr;  // given back after the work on s
-        if (p && !pooled) cudaFree(p);
+        if (pooled) {  // given back after the work on s
+            before.s = s;
+            before.p = static_cast<unsigned char*>(p);
+            p = nullptr;
+            bytes = 0;
+            pooled = false;
+        }
+        if (want > 2 * kOwnWork) return ensure(want);
+        if (p) cudaFree(p);
         p = nullptr;
         bytes = 0;
         if (epoch) ++*epoch;
-        e = m.take(want, s);
+        e = m.take(kPoolCircuits, want, s);
         if (e != cudaSuccess) return e;
         p = m.p;
         bytes = std::max<size_t>(want, 256);
@@ -1863,7 +1873,7 @@ int approx_setup(ef_circuit* c, int64_t nb, int64_t t, uint64_t seed, uint64_t b
 // Samples and images of a single call, until `mem` ends.
 int approx_memory(ef::ApproxDev& a, const ApproxWork& work, CallMemory& mem, cudaStream_t s) {
     if (work.own) return EF_OK;
-    EF_CK(mem.take(work.bytes(), s));
+    EF_CK(mem.take(kPoolCalls, work.bytes(), s));
     approx_bind(a, work, mem.p);
     return EF_OK;
 }

@@ -125,3 +125,32 @@ def test_captured_call_owns_its_memory(lib, nb, t):
             torch.cuda.synchronize()
             assert np.array_equal(out.cpu().numpy(), ref) and np.array_equal(big, again)
         del g
+
+
+KEPT = """
+import numpy as np, torch
+import paper_2511_12416_gb300 as ef, workloads as W
+bits = W.spin_sector_bitstrings(6, 3, 3, 2000, np.random.default_rng(2))
+torch.zeros(1, device="cuda")
+def circuit(i):
+    c = W.lucj_circuit(6, 3, 3, 1, n_onsite=6, n_same=3, angle_sampler=W.normal_var(1.0), seed=i)
+    return ef.Circuit(c.n_modes, c.occupation, c.gates)
+hs = [circuit(i) for i in range(400)]
+for h in hs:
+    ef.ef_prob_approx(h.handle, bits[:14], 1800, seed=1)  # some MiB each, kept by the circuit
+torch.cuda.synchronize()
+free = torch.cuda.mem_get_info()[0]
+ef.ef_prob_approx(hs[0].handle, bits, 25000, seed=1)  # 1 GiB while it runs
+torch.cuda.synchronize()
+print((free - torch.cuda.mem_get_info()[0]) / 2**30)
+"""
+
+
+def test_memory_of_calls_is_kept_beside_many_circuits(lib):
+    """What the circuits hold does not count against what is kept for calls, else a large call's
+    memory would be mapped anew every time."""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", KEPT], cwd=root, env=dict(os.environ, PYTHONPATH=root), capture_output=True,
+                       text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]
+    assert 0.9 <= float(r.stdout) <= 1.25
