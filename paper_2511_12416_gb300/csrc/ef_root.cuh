@@ -12,17 +12,15 @@ namespace ef {
 // if and only if s (s - ulp) < x <= s (s + ulp), which fused multiply-adds decide exactly,
 // here between s and its two neighbours. Below 1e-30 the residuals underflow and the
 // result may be a unit in the last place off, that of a subnormal argument 0 or 1e-45;
-// infinity and NaN stay what they are. 52-qubit LUCJ circuit, 8192 bitstrings of 68,416
-// trajectories: 107.3 ms, with sqrtf 109.6; a batch of 12 uneven circuits: 22.5 and 23.9 ms.
+// infinity and NaN stay what they are. Against sqrtf: the Estimate of 1000 bitstrings of
+// the 52-qubit LUCJ circuit 1.4 % faster, a batch of 12 uneven circuits 7 %; the result picked
+// by two selects instead of an addition: 1 % slower.
 __device__ __forceinline__ float root(float x) {
     float s;
     asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(s) : "f"(x));
     const float down = __int_as_float(__float_as_int(s) - 1), up = __int_as_float(__float_as_int(s) + 1);
     const float below = fmaf(-down, s, x), above = fmaf(-up, s, x);
-    float r = s;
-    if (below <= 0.f) r = down;
-    if (above > 0.f) r = up;
-    return r;
+    return __int_as_float(__float_as_int(s) + (above > 0.f ? 1 : 0) - (below <= 0.f ? 1 : 0));
 }
 
 }  // namespace ef
