@@ -370,7 +370,8 @@ def bench_config3(ef, torch, dev, stream, flush, pool, peaks):
            "trajectories_per_s": traj_s, "fp64_recomputed": st["fp64_recomputed"],
            "sampled_flips": st["sampled_flips"], "max_est_rel_err": float(np.max(np.abs(err))),
            "dominant_kernel_ms": kern_ms,
-           "roofline": {"bound": "alu", "kernel": "k_approx (Philox4x32-10 sampling, one word per gate)",
+           "roofline": {"bound": "alu", "kernel": "k_approx_sample (Philox4x32-10, one word per gate) with the set-up and "
+                                                    "evaluation kernels beside and after it",
                         "achieved": achieved, "peak": peaks["philox_blocks_per_s"], "unit": "Philox blocks/s",
                         "frac": achieved / peaks["philox_blocks_per_s"],
                         "peak_source": "measured (ef_measure_peak kind 3) on this GPU",
@@ -520,7 +521,8 @@ def bench_config4(ef, torch, dev, stream, flush, pool, peaks):
                                            f"({sampled} in all) and scaled to its bitstring count"},
            "batched_over_fp64_single": ms64 / per,
            "max_rel_diff_vs_fp64_form": max_rel,
-           "roofline": {"bound": "alu", "kernel": "k_approx of the Raw Estimate circuits (the bulk of the work)",
+           "roofline": {"bound": "alu", "kernel": "k_approx_sample and k_approx of the Raw Estimate circuits (the bulk of "
+                                                    "the work)",
                         "note": "whole-graph time; the Raw Estimate share is measured in config3_lucj52_approx"}}
     if futs:
         errs, walls = [], 0.0

@@ -67,10 +67,14 @@ __device__ __forceinline__ double recip(double m) { return 1.0 / m; }
 __device__ __forceinline__ float min_pivot2(float) { return 1.17549435e-38f; }
 __device__ __forceinline__ double min_pivot2(double) { return 2.2250738585072014e-308; }
 // Pivot key of an FP64 entry: the leading 32 bits of its larger component, which
-// order as integers (the pivot is within a factor sqrt(2) of the largest).
-// Comparing |a|^2 takes the FP64 pipe three instructions an entry, 64 cycles a
-// warp each. For well-conditioned matrices only: where a minor is singular up
-// to rounding its value hangs on the pivots, and the Exact minors keep |a|^2.
+// order as integers. Comparing |a|^2 takes the FP64 pipe three instructions an entry,
+// 64 cycles a warp each. The pivot is within a factor sqrt(2) of the largest entry:
+// partial pivoting with a threshold, where an elimination step grows entries at most
+// 1 + sqrt(2)-fold instead of 2-fold. Where a determinant is singular up to rounding its
+// value hangs on the pivots. The terms det(I + K[N, N]) of a Raw Estimate, sums of order
+// one, do not show that (24 modes, 500 x 5000: 1.5e-15 off 64-bit values, with |a|^2
+// 1.6e-15, at 1586 and 1617 us); Exact probabilities can consist of such minors, and keep
+// |a|^2.
 __device__ __forceinline__ int pivot_key(double2 a) {
     return max(__double2hiint(a.x) & 0x7fffffff, __double2hiint(a.y) & 0x7fffffff);
 }
